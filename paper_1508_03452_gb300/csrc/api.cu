@@ -11,6 +11,7 @@
 
 #include "aux.cuh"
 #include "lbrmhd.h"
+#include "mlp.cuh"
 
 namespace {
 
@@ -1619,8 +1620,8 @@ int lbrmhd_set_mlp_weights(lbrmhd_handle h, const float* d_params)
         h->d_mlp = nullptr;
         return fail(h, LBRMHD_ERR_OOM, "network blob allocation failed");
     }
-    const int rc = lbrmhd_mlp_pack(d_params, h->d_mlp, h->stream);
-    if (rc) return fail(h, rc, "packing the network failed");
+    if (lb::launch_mlp_pack_warp(d_params, h->d_mlp, h->stream) != cudaSuccess)
+        return fail(h, LBRMHD_ERR_CUDA, "packing the network failed");
     h->mlp_set = true;
     runs_changed(h);  // the kernel arguments carry the blob pointer
     return LBRMHD_OK;

@@ -12,7 +12,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <cstring>
 #include <mutex>
 
 #include "lbrmhd.h"
@@ -327,9 +326,19 @@ __global__ void __launch_bounds__(32 * kReduceShares) mlp_reduce_kernel(const fl
 }
 
 // float32 parameters -> bf16 inference blob in fragment order (zero padding)
+// (WARP: the step kernel's own copy, fragments in warp order)
+template <bool WARP>
 __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __restrict__ blob)
 {
-    __nv_bfloat16* W = reinterpret_cast<__nv_bfloat16*>(blob);
+    __nv_bfloat16* B = reinterpret_cast<__nv_bfloat16*>(blob);
+    struct Out {  // element e of the blob in its own order
+        __nv_bfloat16* p;
+        __device__ __nv_bfloat16& operator[](int e) const
+        {
+            return p[WARP ? 4 * mlp_warp_order(e / 4) + e % 4 : e];
+        }
+    };
+    const Out W{B};
     float* bias = reinterpret_cast<float*>(blob + MLPD_NBF16 * 2);
     const int total = MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H + MLPD_NBIAS;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
@@ -360,114 +369,6 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
     }
 }
 
-// Warp order of the blob's weights: 8-byte fragment i of the blob (row r, k-tile
-// kt, lane column group t of its layer) goes where the fragments of the 32 lanes
-// that use them together, for two k-tiles at a time, are consecutive: a warp's
-// load is 512 bytes in a row. In the blob's own order the 8 rows of a fragment
-// lie K * 2 bytes apart, in the same shared-memory banks.
-__device__ __forceinline__ int mlp_warp_order(int i)
-{
-    const int first = i < MLPD_W2 / 4 ? 0 : (i < MLPD_W3 / 4 ? MLPD_W2 / 4 : (i < MLPD_W4 / 4 ? MLPD_W3 / 4 : MLPD_W4 / 4));
-    const int kt_count = first == 0 ? MLP_K1 / 16 : MLP_H / 16;
-    const int j = i - first, t = j % 4, kt = (j / 4) % kt_count, r = j / (4 * kt_count);
-    const int lane = (r % 8) * 4 + t;
-    return first + ((r / 8) * kt_count + (kt & ~1)) * 32 + 2 * lane + (kt & 1);
-}
-
-// The same forward pass with the activations kept in registers: the accumulator
-// fragment of two 8-wide output tiles is, packed to bf16, the A fragment of one
-// 16-wide k-tile of the next layer, so no activation goes through shared memory.
-// A: [m-tile][k-tile][register] of the K inputs; on return the 64 outputs. The
-// weights are in warp order (mlp_warp_order): two k-tiles' fragments of the 32
-// lanes are 512 consecutive bytes, one 16-byte load a lane.
-template <int K>
-__device__ __forceinline__ void mlp_layer_frag(uint32_t (&A)[2][4][4], const __nv_bfloat16* W, const float* bias)
-{
-    const int lane = threadIdx.x & 31, tig = lane & 3;
-    constexpr int KT = K / 16;
-    const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.0f, 0.0f);
-    uint32_t N[2][4][4];
-#pragma unroll
-    for (int np = 0; np < 4; ++np) {  // output tiles 2 np, 2 np + 1: four independent chains of products
-        float acc[2][2][4];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const float2 b = *reinterpret_cast<const float2*>(bias + 8 * (2 * np + q) + 2 * tig);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                acc[q][mt][0] = acc[q][mt][2] = b.x;
-                acc[q][mt][1] = acc[q][mt][3] = b.y;
-            }
-        }
-#pragma unroll
-        for (int kt = 0; kt < KT; kt += 2) {
-            uint4 bw[2];
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-                bw[q] = *reinterpret_cast<const uint4*>(W + (((2 * np + q) * KT + kt) * 32 + 2 * lane) * 4);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const uint32_t b[2] = {h ? bw[q].z : bw[q].x, h ? bw[q].w : bw[q].y};
-#pragma unroll
-                    for (int mt = 0; mt < 2; ++mt) mma_bf16(acc[q][mt], A[mt][kt + h], b);
-                }
-        }
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    const __nv_bfloat162 v =
-                        __hmax2(__floats2bfloat162_rn(acc[q][mt][2 * hh], acc[q][mt][2 * hh + 1]), zero2);
-                    memcpy(&N[mt][np][2 * q + hh], &v, 4);
-                }
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int kt = 0; kt < 4; ++kt)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) A[mt][kt][r] = N[mt][kt][r];
-}
-
-// Forward pass of the warp's 32 rows: `rows` (shared) holds 32 rows of ROW bf16,
-// 20 features then zeros up to 32; `wts` the inference blob in warp order.
-// y[mt]: the accumulator fragment of rows 16 mt.. (columns 0..3 are the outputs:
-// lanes with lane % 4 < 2 hold columns 2 (lane % 4), + 1 of rows lane / 4, + 8).
-template <int ROW>
-__device__ __forceinline__ void mlp_forward_frag(const __nv_bfloat16* rows, const unsigned char* wts, float (&y)[2][4])
-{
-    const int lane = threadIdx.x & 31, tig = lane & 3;
-    const __nv_bfloat16* W = reinterpret_cast<const __nv_bfloat16*>(wts);
-    const float* bias = reinterpret_cast<const float*>(wts + MLPD_NBF16 * 2);
-    uint32_t A[2][4][4];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int kt = 0; kt < 2; ++kt) ldmatrix_x4(A[mt][kt], rows + (16 * mt + (lane & 15)) * ROW + 16 * kt + (lane >> 4) * 8);
-    mlp_layer_frag<MLP_K1>(A, W + MLPD_W1, bias);
-    mlp_layer_frag<MLP_H>(A, W + MLPD_W2, bias + MLP_H);
-    mlp_layer_frag<MLP_H>(A, W + MLPD_W3, bias + 2 * MLP_H);
-    const float2 b = *reinterpret_cast<const float2*>(bias + 3 * MLP_H + 2 * tig);
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-        y[mt][0] = y[mt][2] = b.x;
-        y[mt][1] = y[mt][3] = b.y;
-    }
-#pragma unroll
-    for (int kt = 0; kt < 4; kt += 2) {
-        const uint4 bw = *reinterpret_cast<const uint4*>(W + MLPD_W4 + (kt * 32 + 2 * lane) * 4);
-        const uint32_t b0[2] = {bw.x, bw.y}, b1[2] = {bw.z, bw.w};
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) mma_bf16(y[mt], A[mt][kt], b0);
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) mma_bf16(y[mt], A[mt][kt + 1], b1);
-    }
-}
-
 // Standalone inference: a warp takes 32 rows at a time through the network, the
 // activations staying in its registers from layer to layer (mlp_forward_frag),
 // the weights read from the block's shared copy; same products and sums in the
@@ -478,13 +379,12 @@ __device__ __forceinline__ void mlp_forward_frag(const __nv_bfloat16* rows, cons
 // through shared memory, and the rows and the weight fragments were loaded at
 // strides: L1 92 % busy, 121 us.
 constexpr int kInferWarps = 4, kInferBlocks = 3;  // warps per block, blocks per SM (4: 128 registers spill, 74 us)
-constexpr int kFeatRow = 40;  // bf16 per staged feature row: the 8 rows of an 8x8 fragment in distinct banks
 __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks) mlp_infer_kernel(const unsigned char* __restrict__ blob,
                                                                         const float* __restrict__ feat, int64_t n,
                                                                         float* __restrict__ out)
 {
     __shared__ __align__(16) unsigned char wts[(MLPD_BYTES + 15) / 16 * 16];
-    __shared__ __align__(16) __nv_bfloat16 rows[kInferWarps][32 * kFeatRow];
+    __shared__ __align__(16) __nv_bfloat16 rows[kInferWarps][32 * MLP_FROW];
     const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
     // the blob's fragments (8 bytes a lane), those of a warp's lanes side by side
     for (int i = threadIdx.x; i < MLPD_NBF16 / 4; i += 32 * kInferWarps)
@@ -492,7 +392,7 @@ __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks) mlp_infer_kern
     for (int i = threadIdx.x; i < MLPD_NBIAS; i += 32 * kInferWarps)
         reinterpret_cast<float*>(wts + MLPD_NBF16 * 2)[i] = __ldg(reinterpret_cast<const float*>(blob + MLPD_NBF16 * 2) + i);
     __nv_bfloat16* mine = rows[w];
-    for (int i = lane; i < 32 * kFeatRow; i += 32) mine[i] = __float2bfloat16_rn(0.0f);
+    for (int i = lane; i < 32 * MLP_FROW; i += 32) mine[i] = __float2bfloat16_rn(0.0f);
     __syncthreads();
     constexpr int kVecs = MLP_IN / 4;  // 16-byte vectors per row
     const int64_t ntiles = (n + 31) / 32, total = n * kVecs;
@@ -518,14 +418,14 @@ __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks) mlp_infer_kern
 #pragma unroll
         for (int j = 0; j < kVecs; ++j) {
             const int i = 32 * j + lane;
-            __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(mine + (i / kVecs) * kFeatRow + 4 * (i % kVecs));
+            __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(mine + (i / kVecs) * MLP_FROW + 4 * (i % kVecs));
             p[0] = __floats2bfloat162_rn(f[j].x, f[j].y);
             p[1] = __floats2bfloat162_rn(f[j].z, f[j].w);
         }
         __syncwarp();
         fetch(tile + nw);
         float y[2][4];
-        mlp_forward_frag<kFeatRow>(mine, wts, y);
+        mlp_forward_frag<2, false>(mine, wts, y);
         const int gid = lane >> 2, tig = lane & 3;
         if (tig < 2) {
 #pragma unroll
@@ -541,6 +441,12 @@ __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks) mlp_infer_kern
                 }
         }
     }
+}
+
+cudaError_t launch_mlp_pack_warp(const float* params, unsigned char* blob, cudaStream_t s)
+{
+    mlp_pack_kernel<true><<<32, 256, 0, s>>>(params, blob);
+    return cudaGetLastError();
 }
 
 }  // namespace lb
@@ -652,7 +558,7 @@ int lbrmhd_mlp_blob_bytes(void) { return lb::MLPD_BYTES; }
 int lbrmhd_mlp_pack(const float* d_params, void* d_blob, void* stream)
 {
     if (!d_params || !d_blob) return LBRMHD_ERR_BAD_ARG;
-    lb::mlp_pack_kernel<<<32, 256, 0, (cudaStream_t)stream>>>(d_params, (unsigned char*)d_blob);
+    lb::mlp_pack_kernel<false><<<32, 256, 0, (cudaStream_t)stream>>>(d_params, (unsigned char*)d_blob);
     return cudaGetLastError() == cudaSuccess ? LBRMHD_OK : LBRMHD_ERR_CUDA;
 }
 

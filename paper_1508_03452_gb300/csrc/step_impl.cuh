@@ -501,6 +501,13 @@ struct CollideH<12, Cfg> {
                                                const R*, bool) {}
 };
 
+// 16-row tiles of a warp's 32 cells that the learned seed takes through the network
+// at a time: 1 (231 us a step of the 1024^2 sheet), because two tiles' fragments
+// beside the cell's state spill (239 us) though they read the weights once
+#ifndef LB_MLP_TILES
+#define LB_MLP_TILES 1
+#endif
+constexpr int kMlpTiles = LB_MLP_TILES;
 constexpr int kStepSlots = 63;  // 19 f + 19 g + 25 h pre-collision values per cell in shared memory
 #ifndef LB_STEP_MIN_BLOCKS
 // resident 128-thread blocks per SM targeted for 2-D runs in float32 storage:
@@ -920,16 +927,30 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
     if constexpr (SEED == SEED_MLP) {
         __nv_bfloat16* act =
             reinterpret_cast<__nv_bfloat16*>(smem_raw + (size_t)kStepSlots * sizeof(R) * nth);
-        float* out_f = reinterpret_cast<float*>(smem_raw + (size_t)kStepSlots * sizeof(R) * nth +
-                                                (size_t)MLP_ACT_BYTES_PER_CELL * nth);
-        __nv_bfloat16* row = act + tid * MLP_HS;
+        __nv_bfloat16* row = act + tid * MLP_FROW;
 #pragma unroll
         for (int j = 0; j < 32; j += 2)
             *reinterpret_cast<__nv_bfloat162*>(row + j) =
                 __floats2bfloat162_rn(j < MLP_IN ? feat[j] : 0.0f, j + 1 < MLP_IN ? feat[j + 1] : 0.0f);
         __syncwarp();
-        mlp_forward_warp(act, A.mlp, out_f);
-        R sb[3] = {(R)out_f[tid * 8], (R)out_f[tid * 8 + 1], (R)out_f[tid * 8 + 2]};
+        const int lane = tid & 31;
+#pragma unroll
+        for (int part = 0; part < 2 / kMlpTiles; ++part) {
+            __nv_bfloat16* rows = act + ((tid & ~31) + 16 * kMlpTiles * part) * MLP_FROW;
+            float y[kMlpTiles][4];
+            mlp_forward_frag<kMlpTiles, true>(rows, A.mlp, y);
+            __syncwarp();  // the feature rows have been read: the outputs take their place
+            if ((lane & 3) < 2)
+#pragma unroll
+                for (int mt = 0; mt < kMlpTiles; ++mt)
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh)
+                        *reinterpret_cast<float2*>(rows + (16 * mt + (lane >> 2) + 8 * hh) * MLP_FROW + 4 * (lane & 3)) =
+                            make_float2(y[mt][2 * hh], y[mt][2 * hh + 1]);
+        }
+        __syncwarp();
+        const float* out_f = reinterpret_cast<const float*>(row);
+        R sb[3] = {(R)out_f[0], (R)out_f[1], (R)out_f[2]};
         const R sb2 = sb[0] * sb[0] + sb[1] * sb[1] + sb[2] * sb[2];
         const R lim = R(0.9);  // keep the guess well inside the light cone
         const R scale = sb2 > lim * lim ? lim / sqrt(sb2) : R(1);
@@ -1182,7 +1203,7 @@ template <class Cfg, int NTH = kStepThreads>
 __host__ __device__ constexpr size_t step_cell_smem(int seed)
 {
     return seed == SEED_MLP ? (size_t)kStepSlots * sizeof(typename Cfg::real) * NTH +
-                                  (size_t)(MLP_ACT_BYTES_PER_CELL + 8 * sizeof(float)) * NTH
+                                  (size_t)MLP_ACT_BYTES_PER_CELL * NTH
                             : (size_t)kStepSlots * sizeof(typename Cfg::real) * NTH;
 }
 
