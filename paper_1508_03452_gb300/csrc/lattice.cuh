@@ -97,13 +97,32 @@ struct Prim {
 template <class R>
 __device__ __forceinline__ R sq(R a) { return a * a; }
 
+// a product that is rounded on its own in float64 (never fused into a following
+// sum), where a sum of several products leaves the compiler a choice of which to
+// fuse: every float64 kernel variant then rounds alike
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return a * b; }
+
 __device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
 
 // 1/x where a few ulp do not matter (a relaxation factor, a spectral shift):
 // the hardware reciprocal approximation in float32, the division in float64
 __device__ __forceinline__ float rcp_approx(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double rcp_approx(double x) { return 1.0 / x; }
+// float64: Newton's iteration r <- r + r (1 - x r) from the hardware's 20-bit
+// approximation, twice (a relative error of ~1e-16, four FP64 instructions; the
+// IEEE division takes about ten, and the FP64 pipe, two lanes per SM, is what a
+// float64 step is bound by)
+__device__ __forceinline__ double rcp_approx(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+// 1/x of results: IEEE in float32, the Newton form in float64
+__device__ __forceinline__ float rcp_result(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_result(double x) { return rcp_approx(x); }
 
 // ---------------------------------------------------------------------------
 // equilibria in deviation form (restated from Eq. Dis_fun_EM with the
@@ -121,6 +140,12 @@ __device__ __forceinline__ double rcp_approx(double x) { return 1.0 / x; }
 //   g_i^eq = w'_i n g (1 + 3 q c.b + 4.5 q^2 (c.b)^2 - 1.5 b^2)
 // (b = u / c, g = Lorentz factor, c = chat_i)
 // ---------------------------------------------------------------------------
+// Lorentz factor g of a cell's velocity, g^2 and g - 1
+template <class R>
+struct Lorentz {
+    R g, g2, gm1;
+};
+
 // Per-cell terms of the equilibria. With chat_i having one (axis a, sign s) or
 // two (axes a < b, signs s_a, s_b) non-zero components:
 //   f^eq - W = w_i (even + s odd_a)                                    axis
@@ -136,17 +161,18 @@ struct EqCell {
     R kf, kq[3];
 };
 
+// (lz: the Lorentz factor where the caller has it, else it is formed here)
 // n_dev = n - n_r, eps_dev = eps - eps_r, dE = E - Er and dB = B - Br are passed
 // separately so that the float32 path never rounds the large reference values
 // into the deviations.
 template <class R>
 __device__ __forceinline__ void eq_cell(const Prim<R>& s, R n_dev, R eps_dev, const R* dE, const R* dB,
-                                        const Phys<R>& k, EqCell<R>& q)
+                                        const Phys<R>& k, EqCell<R>& q, const Lorentz<R>* lz = nullptr)
 {
     const R b[3] = {s.u[0] * k.inv_c, s.u[1] * k.inv_c, s.u[2] * k.inv_c};
     const R b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-    const R g2 = R(1) / (R(1) - b2);
-    const R g = sqrt(g2);
+    const R g2 = lz ? lz->g2 : R(1) / (R(1) - b2);
+    const R g = lz ? lz->g : sqrt(g2);
     const R p_dev = k.gm1 * (eps_dev - n_dev * k.c2);
     const R three_dp = R(3) * p_dev;
     const R rest_dev = R(kRest) * (R(3) * p_dev - eps_dev);
@@ -180,7 +206,8 @@ __device__ __forceinline__ void eq_cell(const Prim<R>& s, R n_dev, R eps_dev, co
     }
     const R ng = s.n * g;
     // n g - n_r = n_dev g + n_r (g - 1), g - 1 = g^2 b^2 / (g + 1)
-    const R dng = n_dev * g + k.n_r * (g2 * b2 / (g + R(1)));
+    const R gm1 = lz ? lz->gm1 : g2 * b2 / (g + R(1));
+    const R dng = n_dev * g + mul_rn(k.n_r, gm1);
     q.g_base = dng - R(1.5) * ng * b2;
     for (int a = 0; a < 3; ++a) {
         q.g_lin[a] = R(3) * R(kQ) * ng * b[a];
@@ -316,7 +343,7 @@ __device__ __forceinline__ void ohm_solve(const R* Ep, const R* u, const R* B, R
     const R hs = k.half_dt_c2 * k.sigma;
     const R kk = hs * g;
     const R kg = R(1) + hs * ig;  // 1 + k/g^2
-    const R inv = R(1) / ((R(1) + kk) * kg);
+    const R inv = rcp_result((R(1) + kk) * kg);
     const R inv1k = kg * inv;
     const R kfrac = kk * inv1k;
     R a[3];

@@ -35,6 +35,19 @@ __device__ __forceinline__ R minmod(R a, R b)
     return fmax(fmin(a, b), fmin(fmax(a, b), R(0)));
 }
 
+// the same in float64, chosen by integer compares of the bit patterns (magnitudes
+// of doubles order like their bits): a float64 min or max takes the FP64 pipe,
+// which bounds the float64 step (two lanes per SM), the integer pipes are idle.
+// An argument that is not a number gives the other one, as fmin / fmax do.
+__device__ __forceinline__ double minmod(double a, double b)
+{
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+    const long long ma = ia & 0x7fffffffffffffffll, mb = ib & 0x7fffffffffffffffll;
+    const bool a_less = ma <= mb;
+    const bool opposite = (ia ^ ib) < 0 && (a_less ? mb : ma) <= 0x7ff0000000000000ll;
+    return __longlong_as_double(opposite ? 0ll : (a_less ? ia : ib));
+}
+
 template <class R>
 __device__ __forceinline__ R flux_diff(R um2, R um1, R u0, R up1, R kappa)
 {
@@ -122,6 +135,68 @@ __device__ __forceinline__ void acc_fg_pair(R fI, R gI, R fJ, R gJ, R (&Tm)[10],
     if (cz) Na[2] += R(cz) * dg;
 }
 
+// stream_group in float64, where the number of FP64 instructions is the time: the
+// differences along an axis are formed once for the flux and the Laplacian, the
+// sums over axes start from their first term, and the Courant number multiplies
+// the summed flux once. (326 FP64 instructions per cell of a 2-D run against
+// ~720 of the float32 form with its minima and maxima.)
+template <int G, bool IS3D, class Ld>
+__device__ __forceinline__ V4<double> stream_group_f64(const V4<double>& v, const Ld& ld, const Phys<double>& k)
+{
+    constexpr int I = 2 * G - 1;
+    constexpr int s[3] = {c19(I, 0), c19(I, 1), c19(I, 2)};
+    constexpr int first_move = s[0] != 0 ? 0 : (s[1] != 0 ? 1 : 2);  // the first axis with a flux
+    constexpr int still = (s[0] == 0) + (s[1] == 0) + (IS3D && s[2] == 0);
+    constexpr bool moves = s[0] != 0 || s[1] != 0 || (IS3D && s[2] != 0);
+    double S[4] = {0, 0, 0, 0}, M[4] = {0, 0, 0, 0};  // sums of the first-order and the limited differences
+    double L[2] = {0, 0}, Q[2] = {0, 0};              // Laplacian of f: moving axes; neighbour sums of the others
+    bool q_first = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (a == 2 && !IS3D) continue;
+        if (s[a] != 0) {
+            const V4<double> m2 = ld(a, -2), m1 = ld(a, -1), p1 = ld(a, 1), p2 = ld(a, 2);
+            const V4<double>& i2 = s[a] > 0 ? m2 : p2;
+            const V4<double>& i1 = s[a] > 0 ? m1 : p1;
+            const V4<double>& ip = s[a] > 0 ? p1 : m1;
+            const V4<double>& j2 = s[a] > 0 ? p2 : m2;
+            const double d0[4] = {v.x - i1.x, v.y - i1.y, v.z - ip.z, v.w - ip.w};
+            const double dp[4] = {ip.x - v.x, ip.y - v.y, i1.z - v.z, i1.w - v.w};
+            const double dm[4] = {i1.x - i2.x, i1.y - i2.y, ip.z - j2.z, ip.w - j2.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double m = minmod(dp[j], d0[j]) - minmod(d0[j], dm[j]);
+                S[j] = a == first_move ? d0[j] : S[j] + d0[j];
+                M[j] = a == first_move ? m : M[j] + m;
+            }
+            L[0] = a == first_move ? dp[0] - d0[0] : L[0] + (dp[0] - d0[0]);
+            L[1] = a == first_move ? dp[2] - d0[2] : L[1] + (dp[2] - d0[2]);
+        } else {
+            const V4<double> m1 = ld(a, -1), p1 = ld(a, 1);
+            const double q0 = m1.x + p1.x, q1 = m1.z + p1.z;
+            Q[0] = q_first ? q0 : Q[0] + q0;
+            Q[1] = q_first ? q1 : Q[1] + q1;
+            q_first = false;
+        }
+    }
+    if constexpr (still > 0) {
+        const double l0 = fma(-2.0 * still, v.x, Q[0]), l1 = fma(-2.0 * still, v.z, Q[1]);
+        L[0] = moves ? L[0] + l0 : l0;
+        L[1] = moves ? L[1] + l1 : l1;
+    }
+    V4<double> out = v;
+    if constexpr (moves) {
+        const double Ck = k.C * k.kappa;
+        out.x = fma(-Ck, M[0], fma(-k.C, S[0], v.x));
+        out.y = fma(-Ck, M[1], fma(-k.C, S[1], v.y));
+        out.z = fma(-Ck, M[2], fma(-k.C, S[2], v.z));
+        out.w = fma(-Ck, M[3], fma(-k.C, S[3], v.w));
+    }
+    out.x = fma(k.kvisc, L[0], out.x);
+    out.z = fma(k.kvisc, L[1], out.z);
+    return out;
+}
+
 // The four streamed populations of fluid group G (pre-collision values at
 // t + dt of f_I, g_I, f_J, g_J for the opposite directions I = 2G-1, J = 2G);
 // ld(a, d) gives the group's 4-vector of the cell d cells away along axis a
@@ -139,6 +214,7 @@ __device__ __forceinline__ V4<typename Cfg::real> stream_group(const Ld& ld, con
     constexpr int I = 2 * G - 1, J = 2 * G;
     constexpr int s[3] = {c19(I, 0), c19(I, 1), c19(I, 2)};
     const V4<R> v0 = ld(0, 0);
+    if constexpr (sizeof(R) == 8) return stream_group_f64<G, IS3D>(v0, ld, k);
     R fl[4] = {R(0), R(0), R(0), R(0)}, lap[2] = {R(0), R(0)};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -374,6 +450,25 @@ __device__ __forceinline__ void acc_h(R hv, R (&dEp)[3], R (&bn)[3], R& rho)
     bn[plane_normal(p)] += R(-se * plane_orient(p)) * hv;  // b_{i0} = -o_p, b_{i1} = +o_p
 }
 
+// both populations of pair M (2M, 2M + 1): in float64 from their sum and
+// difference (6 FP64 instructions instead of 8), in float32 one by one (the
+// pair form ran 0.3 % slower)
+template <int M, class R>
+__device__ __forceinline__ void acc_h_pair(R h0, R h1, R (&dEp)[3], R (&bn)[3], R& rho)
+{
+    constexpr int K = 2 * M, p = K / 8, i = (K % 8) / 2, ie = (i + 3) % 4;
+    if constexpr (sizeof(R) == 8) {
+        const R d = h0 - h1;
+        rho += h0 + h1;
+        dEp[plane_a1(p)] += R(hop_s1(ie)) * d;
+        dEp[plane_a2(p)] += R(hop_s2(ie)) * d;
+        bn[plane_normal(p)] += R(-plane_orient(p)) * d;
+    } else {
+        acc_h<K>(h0, dEp, bn, rho);
+        acc_h<K + 1>(h1, dEp, bn, rho);
+    }
+}
+
 template <int M, bool IS3D, class Cfg>
 struct PullH {
     using R = typename Cfg::real;
@@ -385,8 +480,7 @@ struct PullH {
         if (IS3D) off += o.z[2 - hop13(K, 2)];
         const V2<R> hv = ld_hpair<Cfg>(A.hin + h_elem(K, c + off, A.stride));
         put_pair<R, Cfg::kVecSlots>(S.h(K), S.h(K + 1), hv.x, hv.y);
-        acc_h<K>(hv.x, dEp, bn, rho);
-        acc_h<K + 1>(hv.y, dEp, bn, rho);
+        acc_h_pair<M>(hv.x, hv.y, dEp, bn, rho);
         PullH<M + 1, IS3D, Cfg>::run(A, o, c, S, dEp, bn, rho);
     }
 };
@@ -447,6 +541,91 @@ __device__ __forceinline__ void collide_fg(const StepArgs<Cfg>& A, typename Cfg:
     }
 }
 
+// Terms of the float64 collision, the direction weights taken in: f^eq of the
+// opposite directions +-c is E +- O with E even and O odd in c, and so is g^eq
+// (198 FP64 instructions per cell instead of 237 direction by direction).
+struct EqEven {
+    double f0, g0;                         // rest pair
+    double fe_ax[3], fo_ax[3], fe_dg[3], fo_dg[3], fx[3];
+    double ge_ax[3], go_ax[3], ge_dg[3], go_dg[3], gx[3];
+    double kf, kq[3];
+};
+__device__ __forceinline__ void eq_even(const EqCell<double>& q, EqEven& e)
+{
+    constexpr double wa = w19(1), wd = w19(7), va = wg19(1), vd = wg19(7);
+    e.f0 = mul_rn(w19(0), q.f_rest);
+    e.g0 = mul_rn(wg19(0), q.g_base);
+    double base[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        base[a] = q.g_base + q.g_sq[a];
+        e.fe_ax[a] = mul_rn(wa, q.f_even_ax[a]);
+        e.fo_ax[a] = mul_rn(wa, q.f_odd[a]);
+        e.fo_dg[a] = mul_rn(wd, q.f_odd[a]);
+        e.ge_ax[a] = mul_rn(va, base[a]);
+        e.go_ax[a] = mul_rn(va, q.g_lin[a]);
+        e.go_dg[a] = mul_rn(vd, q.g_lin[a]);
+        e.kq[a] = q.kq[a];
+    }
+    e.kf = q.kf;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        e.fe_dg[m] = mul_rn(wd, q.f_even_dg[m]);
+        e.fx[m] = mul_rn(wd, q.f_cross[m]);
+        e.ge_dg[m] = mul_rn(vd, (base[m == 2 ? 1 : 0] + q.g_sq[m == 0 ? 1 : 2]));
+        e.gx[m] = mul_rn(vd, q.g_x[m]);
+    }
+}
+
+// post-collision f and g of group G (directions I = 2G - 1 and -I) from the streamed ones
+template <int G>
+__device__ __forceinline__ V4<double> collide_even(const EqEven& e, const V4<double>& d, double inv_tau)
+{
+    constexpr int I = 2 * G - 1, a = ax1(I), b = ax2(I);
+    double fe, fo, ge, go, ko;
+    if constexpr (b < 0) {
+        static_assert(c19(I, a) == 1, "the first direction of an axis group points along it");
+        fe = e.fe_ax[a], fo = e.fo_ax[a], ge = e.ge_ax[a], go = e.go_ax[a], ko = e.kq[a];
+    } else {
+        constexpr int m = a + b - 1;
+        constexpr double sb = c19(I, b);
+        static_assert(c19(I, a) == 1, "the first direction of a diagonal group points along its first axis");
+        fe = e.fe_dg[m] + sb * e.fx[m];
+        fo = e.fo_dg[a] + sb * e.fo_dg[b];
+        ge = e.ge_dg[m] + sb * e.gx[m];
+        go = e.go_dg[a] + sb * e.go_dg[b];
+        ko = e.kq[a] + sb * e.kq[b];
+    }
+    V4<double> v;
+    v.x = fma(ko - e.kf, d.x - (fe + fo), d.x);
+    v.y = fma(-inv_tau, d.y - (ge + go), d.y);
+    v.z = fma(-(ko + e.kf), d.z - (fe - fo), d.z);
+    v.w = fma(-inv_tau, d.w - (ge - go), d.w);
+    return v;
+}
+
+template <int G>
+struct CollideEven {
+    static __device__ __forceinline__ void run(const StepArgs<CfgF64>& A, int64_t c, const CfgSlots<CfgF64>& S,
+                                               const EqEven& e)
+    {
+        if constexpr (G == 0) {
+            const V2<double> d = get_pair<double, CfgF64::kVecSlots>(S.f(0), S.g(0));
+            st_fgpair<CfgF64>(A.fgout + fg_elem(0, 0, c, A.stride), fma(-e.kf, d.x - e.f0, d.x),
+                              fma(-A.k.inv_tau, d.y - e.g0, d.y), 1.0f, 1.0f);
+        } else {
+            st_quad<CfgF64>(A.fgout + fg_elem(2 * G - 1, 0, c, A.stride),
+                            collide_even<G>(e, get_group(S, G), A.k.inv_tau), V4<float>{1.0f, 1.0f, 1.0f, 1.0f});
+        }
+        CollideEven<G + 1>::run(A, c, S, e);
+    }
+};
+template <>
+struct CollideEven<kFGroups + 1> {
+    static __device__ __forceinline__ void run(const StepArgs<CfgF64>&, int64_t, const CfgSlots<CfgF64>&,
+                                               const EqEven&) {}
+};
+
 // Collision of f and g and the stores, group by group (G onwards) into cell c
 // of the output buffer.
 template <int G, class Cfg>
@@ -478,28 +657,32 @@ struct CollideFG<kFGroups + 1, Cfg> {
     static __device__ __forceinline__ void run(const StepArgs<Cfg>&, int64_t, const CfgSlots<Cfg>&, const EqCell<R>&) {}
 };
 
-// Collision of the Maxwell pair (2M, 2M + 1) into cell c of the output buffer.
-template <int M, class Cfg>
-struct CollideH {
+// Collision of the Maxwell populations of plane P (pairs 4P..4P + 3), h -> 2 h^eq - h,
+// into cell c of the output buffer: with a1, a2 the plane's axes, 2 h^eq of pair i is
+// 2a +- (2e - 2m), 2a and 2e being +-(sum or difference) of the two scaled components
+// of J and E (24 additions per plane).
+template <int P, class Cfg>
+__device__ __forceinline__ void collide_h_plane(const StepArgs<Cfg>& A, int64_t c, const CfgSlots<Cfg>& S,
+                                                const typename Cfg::real* E, const typename Cfg::real* B,
+                                                const typename Cfg::real* J, bool em_coll)
+{
     using R = typename Cfg::real;
-    static __device__ __forceinline__ void run(const StepArgs<Cfg>& A, int64_t c, const CfgSlots<Cfg>& S, const R* E,
-                                               const R* B, const R* J, bool em_coll)
-    {
-        constexpr int K = 2 * M;
-        const V2<R> hs = get_pair<R, Cfg::kVecSlots>(S.h(K), S.h(K + 1));
-        const R h0 = hs.x, h1 = hs.y;
-        const R v0 = em_coll ? R(2) * heq13<K>(E, B, J, A.k) - h0 : h0;
-        const R v1 = em_coll ? R(2) * heq13<K + 1>(E, B, J, A.k) - h1 : h1;
+    constexpr int a1 = plane_a1(P), a2 = plane_a2(P);
+    const R js = R(kSqrt2 / 8.0) * A.k.c, es = R(kSqrt2 / 8.0) * A.k.inv_c;
+    const R j1 = mul_rn(js, J[a1]), j2 = mul_rn(js, J[a2]), e1 = mul_rn(es, E[a1]), e2 = mul_rn(es, E[a2]);
+    const R m = mul_rn(R(0.25 * plane_orient(P)), B[plane_normal(P)]);
+    const R jp = j1 + j2, jm = j1 - j2, ep = e1 + e2, em = e1 - e2;
+    // hops (+,+), (-,+), (-,-), (+,-); the e of pair i lies along hop i - 1
+    const R a[4] = {jp, -jm, -jp, jm}, x[4] = {em - m, ep - m, -em - m, -ep - m};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int K = 8 * P + 2 * i;
+        const V2<R> h = get_pair<R, Cfg::kVecSlots>(S.h(K), S.h(K + 1));
+        const R v0 = em_coll ? (a[i] + x[i]) - h.x : h.x;
+        const R v1 = em_coll ? (a[i] - x[i]) - h.y : h.y;
         st_hpair<Cfg>(A.hout + h_elem(K, c, A.stride), v0, v1);
-        CollideH<M + 1, Cfg>::run(A, c, S, E, B, J, em_coll);
     }
-};
-template <class Cfg>
-struct CollideH<12, Cfg> {
-    using R = typename Cfg::real;
-    static __device__ __forceinline__ void run(const StepArgs<Cfg>&, int64_t, const CfgSlots<Cfg>&, const R*, const R*,
-                                               const R*, bool) {}
-};
+}
 
 // 16-row tiles of a warp's 32 cells that the learned seed takes through the network
 // at a time: 1 (231 us a step of the 1024^2 sheet), because two tiles' fragments
@@ -999,6 +1182,7 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
     landau_b(T, Bc, k, LB);
     Prim<R> nw;
     R J[3], n_dev, eps_dev;
+    Lorentz<R> lz{};  // float64: the recovery's Lorentz factor serves the equilibria too
     int it = 0;
     bool ok = true;
     R d_prev = R(1e30);
@@ -1049,12 +1233,13 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
         const R ed = lambda - s_old;  // eps - eps_r
         const R W = (k.eps_r + k.p_r + ed + k.gm1 * ed) * g2;
         const R kk = k.half_dt_c2 * k.sigma * g;
-        const R q = kk * rcp_approx((R(1) + kk) * W);  // r / B^2
-        const R th = rcp_approx(R(1) + Bn2 * q);
-        const R par = th * q * dB;                      // (1 - th) (dE.B) / B^2
+        const R kW = (R(1) + kk) * W;
+        const R rd = rcp_approx(kW + Bn2 * kk);  // r / B^2 = kk / kW
+        const R th = kW * rd;
+        const R par = kk * rd * dB;              // (1 - th) (dE.B) / B^2
 #pragma unroll
         for (int a = 0; a < 3; ++a) Ec[a] += th * (nw.E[a] - Ec[a]) + par * Bn[a];
-        const R nd = (dN0 - k.n_r * (g2 * b2 * rcp_approx(g + R(1)))) * ig;  // n - n_r
+        const R nd = (dN0 - k.n_r * (g - R(1))) * ig;  // n - n_r, to the digits a spectral shift needs
         p_shift = k.p_r + k.gm1 * (ed - nd * k.c2);
     }
 #pragma unroll
@@ -1062,7 +1247,12 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
     if (ok) {
         eps_dev = lambda - s_old;
         // n = N^0 / U^0: n - n_r = (dN0 - n_r (g - 1)) / g, g - 1 = g^2 b^2 / (g + 1)
-        n_dev = (dN0 - k.n_r * (g2 * b2 / (g + R(1)))) / g;
+        if constexpr (sizeof(R) == 8) {
+            lz = {g, g2, mul_rn(g2 * b2, rcp_approx(g + R(1)))};
+            n_dev = (dN0 - k.n_r * lz.gm1) * ig;
+        } else {
+            n_dev = (dN0 - k.n_r * (g2 * b2 / (g + R(1)))) / g;
+        }
         nw.eps = k.eps_r + eps_dev;
         nw.n = k.n_r + n_dev;
 #pragma unroll
@@ -1135,13 +1325,21 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
 #pragma unroll
     for (int a = 0; a < 3; ++a) dE[a] = nw.E[a] - k.Er[a];
     EqCell<R> q;
-    eq_cell(nw, n_dev, eps_dev, dE, dB, k, q);
+    eq_cell(nw, n_dev, eps_dev, dE, dB, k, q, sizeof(R) == 8 && ok && !relax_eq ? &lz : nullptr);
     if (kOpenCode && relax_eq) SetEqFG<0, Cfg>::run(S, q);
-    CollideFG<0, Cfg>::run(A, c + dco, S, q);
+    if constexpr (sizeof(R) == 8) {
+        EqEven e;
+        eq_even(q, e);
+        CollideEven<0>::run(A, c + dco, S, e);
+    } else {
+        CollideFG<0, Cfg>::run(A, c + dco, S, q);
+    }
     const bool em_coll = (A.flags & FLAG_NO_EM_COLLISION) == 0;
     // h_c - h_ref = 2 h^eq(E - Er, B - Br, J) - (h - h_ref)  (Eq. Maxwell-eq is linear)
     const int64_t co = c + dco;
-    CollideH<0, Cfg>::run(A, co, S, dE, dB, J, em_coll);
+    collide_h_plane<0, Cfg>(A, co, S, dE, dB, J, em_coll);
+    collide_h_plane<1, Cfg>(A, co, S, dE, dB, J, em_coll);
+    collide_h_plane<2, Cfg>(A, co, S, dE, dB, J, em_coll);
     const R h24o = em_coll ? R(2) * nw.rho - *S.h(24) : *S.h(24);
     A.hout[h_elem(24, co, A.stride)] = (typename Cfg::hpop)h24o;
     {
