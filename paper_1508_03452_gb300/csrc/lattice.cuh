@@ -117,8 +117,11 @@ __device__ __forceinline__ double rcp_approx(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
+    // 1/0, 1/inf: the approximation is exact and Newton's product not a number
+    // (told apart by its exponent, on the integer pipe)
+    const bool edge = (((unsigned)__double2hiint(r) & 0x7ff00000u) - 0x00100000u) >= 0x7fe00000u;
+    const double q = fma(r, fma(-x, r, 1.0), r);
+    return edge ? r : fma(q, fma(-x, q, 1.0), q);
 }
 // 1/x of results: IEEE in float32, the Newton form in float64
 __device__ __forceinline__ float rcp_result(float x) { return 1.0f / x; }

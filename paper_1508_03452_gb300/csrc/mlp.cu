@@ -317,11 +317,13 @@ __global__ void __launch_bounds__(32 * kReduceShares) mlp_reduce_kernel(const fl
             if (loss) *loss = g;
             return;
         }
-        const float mi = a.b1 * m[i] + (1.0f - a.b1) * g;
-        const float vi = a.b2 * v[i] + (1.0f - a.b2) * g * g;
+        // from L2: a launch that started early may share its SM with a block of the
+        // step before the last, whose L1 lines of m and v reach into this block's
+        const float mi = a.b1 * __ldcg(m + i) + (1.0f - a.b1) * g;
+        const float vi = a.b2 * __ldcg(v + i) + (1.0f - a.b2) * g * g;
         m[i] = mi;
         v[i] = vi;
-        P[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+        P[i] = __ldcg(P + i) - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
     }
 }
 

@@ -657,10 +657,34 @@ struct CollideFG<kFGroups + 1, Cfg> {
     static __device__ __forceinline__ void run(const StepArgs<Cfg>&, int64_t, const CfgSlots<Cfg>&, const EqCell<R>&) {}
 };
 
-// Collision of the Maxwell populations of plane P (pairs 4P..4P + 3), h -> 2 h^eq - h,
+// Collision of the Maxwell pair (2M, 2M + 1) into cell c of the output buffer.
+template <int M, class Cfg>
+struct CollideH {
+    using R = typename Cfg::real;
+    static __device__ __forceinline__ void run(const StepArgs<Cfg>& A, int64_t c, const CfgSlots<Cfg>& S, const R* E,
+                                               const R* B, const R* J, bool em_coll)
+    {
+        constexpr int K = 2 * M;
+        const V2<R> hs = get_pair<R, Cfg::kVecSlots>(S.h(K), S.h(K + 1));
+        const R h0 = hs.x, h1 = hs.y;
+        const R v0 = em_coll ? R(2) * heq13<K>(E, B, J, A.k) - h0 : h0;
+        const R v1 = em_coll ? R(2) * heq13<K + 1>(E, B, J, A.k) - h1 : h1;
+        st_hpair<Cfg>(A.hout + h_elem(K, c, A.stride), v0, v1);
+        CollideH<M + 1, Cfg>::run(A, c, S, E, B, J, em_coll);
+    }
+};
+template <class Cfg>
+struct CollideH<12, Cfg> {
+    using R = typename Cfg::real;
+    static __device__ __forceinline__ void run(const StepArgs<Cfg>&, int64_t, const CfgSlots<Cfg>&, const R*, const R*,
+                                               const R*, bool) {}
+};
+
+// float64: collision of the Maxwell populations of plane P (pairs 4P..4P + 3), h -> 2 h^eq - h,
 // into cell c of the output buffer: with a1, a2 the plane's axes, 2 h^eq of pair i is
 // 2a +- (2e - 2m), 2a and 2e being +-(sum or difference) of the two scaled components
-// of J and E (24 additions per plane).
+// of J and E (24 additions per plane). (Float32 keeps the form by population: the
+// rounding of this one moves E past the resolution of the fields in long runs.)
 template <int P, class Cfg>
 __device__ __forceinline__ void collide_h_plane(const StepArgs<Cfg>& A, int64_t c, const CfgSlots<Cfg>& S,
                                                 const typename Cfg::real* E, const typename Cfg::real* B,
@@ -1233,13 +1257,21 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
         const R ed = lambda - s_old;  // eps - eps_r
         const R W = (k.eps_r + k.p_r + ed + k.gm1 * ed) * g2;
         const R kk = k.half_dt_c2 * k.sigma * g;
-        const R kW = (R(1) + kk) * W;
-        const R rd = rcp_approx(kW + Bn2 * kk);  // r / B^2 = kk / kW
-        const R th = kW * rd;
-        const R par = kk * rd * dB;              // (1 - th) (dE.B) / B^2
+        R th, par, nd;  // nd: n - n_r
+        if constexpr (sizeof(R) == 8) {
+            const R kW = (R(1) + kk) * W;
+            const R rd = rcp_approx(kW + Bn2 * kk);  // r / B^2 = kk / kW
+            th = kW * rd;
+            par = kk * rd * dB;              // (1 - th) (dE.B) / B^2
+            nd = (dN0 - k.n_r * (g - R(1))) * ig;  // to the digits a spectral shift needs
+        } else {
+            const R q = kk * rcp_approx((R(1) + kk) * W);  // r / B^2
+            th = rcp_approx(R(1) + Bn2 * q);
+            par = th * q * dB;                      // (1 - th) (dE.B) / B^2
+            nd = (dN0 - k.n_r * (g2 * b2 * rcp_approx(g + R(1)))) * ig;
+        }
 #pragma unroll
         for (int a = 0; a < 3; ++a) Ec[a] += th * (nw.E[a] - Ec[a]) + par * Bn[a];
-        const R nd = (dN0 - k.n_r * (g - R(1))) * ig;  // n - n_r, to the digits a spectral shift needs
         p_shift = k.p_r + k.gm1 * (ed - nd * k.c2);
     }
 #pragma unroll
@@ -1337,9 +1369,13 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
     const bool em_coll = (A.flags & FLAG_NO_EM_COLLISION) == 0;
     // h_c - h_ref = 2 h^eq(E - Er, B - Br, J) - (h - h_ref)  (Eq. Maxwell-eq is linear)
     const int64_t co = c + dco;
-    collide_h_plane<0, Cfg>(A, co, S, dE, dB, J, em_coll);
-    collide_h_plane<1, Cfg>(A, co, S, dE, dB, J, em_coll);
-    collide_h_plane<2, Cfg>(A, co, S, dE, dB, J, em_coll);
+    if constexpr (sizeof(R) == 8) {
+        collide_h_plane<0, Cfg>(A, co, S, dE, dB, J, em_coll);
+        collide_h_plane<1, Cfg>(A, co, S, dE, dB, J, em_coll);
+        collide_h_plane<2, Cfg>(A, co, S, dE, dB, J, em_coll);
+    } else {
+        CollideH<0, Cfg>::run(A, co, S, dE, dB, J, em_coll);
+    }
     const R h24o = em_coll ? R(2) * nw.rho - *S.h(24) : *S.h(24);
     A.hout[h_elem(24, co, A.stride)] = (typename Cfg::hpop)h24o;
     {
