@@ -70,6 +70,127 @@ struct HeqStore<24, Cfg, R> {
                                                const Phys<R>&) {}
 };
 
+// Conversions between float32 and float64 on the integer pipes, the same values as
+// the conversion instructions: those share GB300's float64 pipe (two lanes per SM),
+// which bounds the passes below. Zeros and normal numbers are converted by shifts;
+// what is left (subnormals, infinities, NaN, overflow) takes the instruction.
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    return m == 0u ? __hiloint2double((int)u, 0) : (double)v;
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+template <class T>
+__device__ __forceinline__ T narrow(double v);
+template <>
+__device__ __forceinline__ double narrow<double>(double v)
+{
+    return v;
+}
+template <>
+__device__ __forceinline__ float narrow<float>(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned hi = (unsigned)(b >> 32), e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 254u) {  // a normal float32: round to nearest even at bit 29, move the exponent
+        const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+        return __uint_as_float((hi & 0x80000000u) | (((unsigned)(r >> 29) - 0xc0000000u) & 0x7fffffffu));
+    }
+    return (b << 1) == 0ull ? __uint_as_float(hi) : (float)v;
+}
+
+// post-equilibrium f and g of the opposite directions of group G, float64 terms
+template <int G, class Cfg>
+struct EqStoreEven {
+    static __device__ __forceinline__ void run(const PopView<Cfg>& V, int64_t c, const EqEven& e)
+    {
+        using R = typename Cfg::real;
+        if constexpr (G == 0) {
+            st_fgpair<Cfg>(V.fg + fg_elem(0, 0, c, V.stride), narrow<R>(e.f0), narrow<R>(e.g0), V.hs.finv[0], V.hs.ginv[0]);
+        } else {
+            constexpr int I = 2 * G - 1, a = ax1(I), b = ax2(I);
+            static_assert(c19(I, a) == 1, "the first direction of a group points along its first axis");
+            double fe, fo, ge, go;
+            if constexpr (b < 0) {
+                fe = e.fe_ax[a], fo = e.fo_ax[a], ge = e.ge_ax[a], go = e.go_ax[a];
+            } else {
+                constexpr int m = a + b - 1;
+                constexpr double sb = c19(I, b);
+                fe = e.fe_dg[m] + sb * e.fx[m];
+                fo = e.fo_dg[a] + sb * e.fo_dg[b];
+                ge = e.ge_dg[m] + sb * e.gx[m];
+                go = e.go_dg[a] + sb * e.go_dg[b];
+            }
+            st_quad<Cfg>(V.fg + fg_elem(I, 0, c, V.stride),
+                         V4<R>{narrow<R>(fe + fo), narrow<R>(ge + go), narrow<R>(fe - fo), narrow<R>(ge - go)},
+                         V4<float>{V.hs.finv[I], V.hs.ginv[I], V.hs.finv[I + 1], V.hs.ginv[I + 1]});
+        }
+        EqStoreEven<G + 1, Cfg>::run(V, c, e);
+    }
+};
+template <class Cfg>
+struct EqStoreEven<kFGroups + 1, Cfg> {
+    static __device__ __forceinline__ void run(const PopView<Cfg>&, int64_t, const EqEven&) {}
+};
+
+// h^eq of plane P's pairs, float64: a +- (e - m), a and e being +-(sum or difference)
+// of the two scaled components of J and E
+template <int P, class Cfg>
+__device__ __forceinline__ void heq_store_plane(const PopView<Cfg>& V, int64_t c, const double* E, const double* B,
+                                                const double* J, const Phys<double>& k)
+{
+    constexpr int a1 = plane_a1(P), a2 = plane_a2(P);
+    const double js = kSqrt2 / 16.0 * k.c, es = kSqrt2 / 16.0 * k.inv_c;
+    const double j1 = js * J[a1], j2 = js * J[a2], e1 = es * E[a1], e2 = es * E[a2];
+    const double m = 0.125 * plane_orient(P) * B[plane_normal(P)];
+    const double jp = j1 + j2, jm = j1 - j2, ep = e1 + e2, em = e1 - e2;
+    // hops (+,+), (-,+), (-,-), (+,-); the e of pair i lies along hop i - 1
+    const double a[4] = {jp, -jm, -jp, jm}, x[4] = {em - m, ep - m, -em - m, -ep - m};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        st_hpair<Cfg>(V.h + h_elem(8 * P + 2 * i, c, V.stride), narrow<typename Cfg::real>(a[i] + x[i]),
+                      narrow<typename Cfg::real>(a[i] - x[i]));
+}
+
+// J from Eq. Ohm in float64, g the Lorentz factor
+__device__ __forceinline__ void ohm_current_g(const double* E, const double* u, const double* B, double rho, double g,
+                                              const Phys<double>& k, double* J)
+{
+    const double sg = k.sigma * g;
+    const double Eu = (E[0] * u[0] + E[1] * u[1] + E[2] * u[2]) * (k.inv_c * k.inv_c);
+    const double F[3] = {fma(u[1], B[2], fma(-u[2], B[1], E[0])), fma(u[2], B[0], fma(-u[0], B[2], E[1])),
+                         fma(u[0], B[1], fma(-u[1], B[0], E[2]))};
+    for (int a = 0; a < 3; ++a) J[a] = fma(rho, u[a], sg * fma(-Eu, u[a], F[a]));
+}
+
+// every population of cell c at its equilibrium for float64 primitives s
+template <class Cfg>
+__device__ __forceinline__ void set_equilibrium_f64(const PopView<Cfg>& V, int64_t c, const Prim<double>& s,
+                                                    const Phys<double>& k)
+{
+    const double b2 = (s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2]) * (k.inv_c * k.inv_c);
+    Lorentz<double> lz;
+    lz.g = rsqrt_newton(1.0 - b2);
+    lz.g2 = lz.g * lz.g;
+    lz.gm1 = lz.g2 * b2 * rcp_approx(lz.g + 1.0);
+    double J[3];
+    ohm_current_g(s.E, s.u, s.B, s.rho, lz.g, k, J);
+    const double dE[3] = {s.E[0] - k.Er[0], s.E[1] - k.Er[1], s.E[2] - k.Er[2]};
+    const double dB[3] = {s.B[0] - k.Br[0], s.B[1] - k.Br[1], s.B[2] - k.Br[2]};
+    EqCell<double> q;
+    eq_cell(s, s.n - k.n_r, s.eps - k.eps_r, dE, dB, k, q, &lz);
+    EqEven e;
+    eq_even(q, e);
+    EqStoreEven<0, Cfg>::run(V, c, e);
+    heq_store_plane<0, Cfg>(V, c, dE, dB, J, k);
+    heq_store_plane<1, Cfg>(V, c, dE, dB, J, k);
+    heq_store_plane<2, Cfg>(V, c, dE, dB, J, k);
+    V.h[h_elem(24, c, V.stride)] = narrow<typename Cfg::hpop>(s.rho);
+}
+
 // every population of cell c at its equilibrium for primitives s (the
 // post-collision value of an equilibrium state is the equilibrium itself)
 template <class Cfg, class R>
@@ -104,8 +225,22 @@ __device__ __forceinline__ void input_E(const InitInputs& in, int64_t c, int64_t
     }
 }
 
+// component A of the input E at cell c
+template <int A>
+__device__ __forceinline__ double input_E1(const InitInputs& in, int64_t c, int64_t N)
+{
+    if (in.E) return in.E[A * N + c];
+    constexpr int p = (A + 1) % 3, q = (A + 2) % 3;
+    return -(in.u[p * N + c] * in.B[q * N + c] - in.u[q * N + c] * in.B[p * N + c]);
+}
+
+// Bound by GB300's float64 rate (two lanes per SM): opposite directions share the
+// even and odd parts of their equilibria, a plane's Maxwell pairs their sums, one
+// Lorentz factor serves J and the equilibria, reciprocals and the square root are
+// Newton's, and results become float32 on the integer pipes.
 template <class Cfg>
-__global__ void init_kernel(PopView<Cfg> V, InitInputs in, Phys<double> k, int* bad)
+__global__ void __launch_bounds__(128) init_kernel(PopView<Cfg> V, InitInputs in, Phys<double> k, double inv_gm1,
+                                                   double eps0_2dx, int* bad)
 {
     const int64_t N = (int64_t)V.nx * V.ny * V.nz;
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -113,28 +248,45 @@ __global__ void init_kernel(PopView<Cfg> V, InitInputs in, Phys<double> k, int* 
     const int x = (int)(c % V.nx), y = (int)((c / V.nx) % V.ny), z = (int)(c / ((int64_t)V.nx * V.ny));
     Prim<double> s;
     s.n = in.n[c];
-    s.eps = s.n * k.c2 + in.p[c] / k.gm1;
+    s.eps = s.n * k.c2 + in.p[c] * inv_gm1;
     for (int a = 0; a < 3; ++a) {
         s.u[a] = in.u[a * N + c];
         s.B[a] = in.B[a * N + c];
     }
     input_E(in, c, N, s.E);
     if (!(s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2] < k.c2) || !(s.n > 0)) atomicExch(bad, 1);
-    const int q[3] = {x, y, z}, n[3] = {V.nx, V.ny, V.nz};
+    // rho_c = eps0 div E
     double div = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        if (n[a] == 1) continue;
-        int qp[3] = {q[0], q[1], q[2]}, qm[3] = {q[0], q[1], q[2]};
-        qp[a] = wrap_coord(q[a] + 1, n[a], V.periodic[a]);
-        qm[a] = wrap_coord(q[a] - 1, n[a], V.periodic[a]);
-        double Ep[3], Em[3];
-        input_E(in, qp[0] + (int64_t)V.nx * (qp[1] + (int64_t)V.ny * qp[2]), N, Ep);
-        input_E(in, qm[0] + (int64_t)V.nx * (qm[1] + (int64_t)V.ny * qm[2]), N, Em);
-        div += (Ep[a] - Em[a]) / (2.0 * k.dx);
+    if (V.nx > 1) {
+        const int64_t row = c - x;
+        div += input_E1<0>(in, row + wrap_coord(x + 1, V.nx, V.periodic[0]), N) -
+               input_E1<0>(in, row + wrap_coord(x - 1, V.nx, V.periodic[0]), N);
     }
-    s.rho = k.eps0 * div;
-    store_prim<Cfg>(V.prim, V.stride, c, s);
-    set_equilibrium<Cfg, double>(V, c, s, k);
+    if (V.ny > 1) {
+        const int64_t col = c - (int64_t)V.nx * y;
+        div += input_E1<1>(in, col + (int64_t)V.nx * wrap_coord(y + 1, V.ny, V.periodic[1]), N) -
+               input_E1<1>(in, col + (int64_t)V.nx * wrap_coord(y - 1, V.ny, V.periodic[1]), N);
+    }
+    if (V.nz > 1) {
+        const int64_t plane = (int64_t)V.nx * V.ny, col = c - plane * z;
+        div += input_E1<2>(in, col + plane * wrap_coord(z + 1, V.nz, V.periodic[2]), N) -
+               input_E1<2>(in, col + plane * wrap_coord(z - 1, V.nz, V.periodic[2]), N);
+    }
+    s.rho = eps0_2dx * div;
+    {
+        typename Cfg::prim pv[NPRIM];
+        pv[P_N] = narrow<typename Cfg::prim>(s.n);
+        pv[P_EPS] = narrow<typename Cfg::prim>(s.eps);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            pv[P_U + a] = narrow<typename Cfg::prim>(s.u[a]);
+            pv[P_E + a] = narrow<typename Cfg::prim>(s.E[a]);
+            pv[P_B + a] = narrow<typename Cfg::prim>(s.B[a]);
+        }
+        pv[P_RHO] = narrow<typename Cfg::prim>(s.rho);
+        st_prims<Cfg>(V.prim + prim_elem(0, c, V.stride), V.stride, pv);
+    }
+    set_equilibrium_f64<Cfg>(V, c, s, k);
 }
 
 // float64 means for the reference state: n, p, E (3), B (3), E_a E_b (6: xx yy
@@ -222,12 +374,14 @@ struct FixF<19, Cfg, R> {
 // nfaces = 1: the face `hi` of axis a; nfaces = 2: both faces of axis a in one
 // launch (independent when the axis has at least 4 cells: a face writes its
 // boundary layer and reads the two layers inside it)
-template <class Cfg>
-__global__ void bfix_kernel(PopView<Cfg> V, Phys<typename Cfg::real> k, int a, int hi_first, int nfaces)
+// (the axis a is a template argument: with indices known at compile time nothing
+// goes through local memory)
+template <class Cfg, int a>
+__global__ void __launch_bounds__(128) bfix_kernel(PopView<Cfg> V, Phys<typename Cfg::real> k, int hi_first, int nfaces)
 {
     using R = typename Cfg::real;
     const int n[3] = {V.nx, V.ny, V.nz};
-    const int a1 = (a + 1) % 3, a2 = (a + 2) % 3;
+    constexpr int a1 = (a + 1) % 3, a2 = (a + 2) % 3;
     const int64_t face = (int64_t)n[a1] * n[a2];
     const int64_t mm = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (mm >= nfaces * face) return;
@@ -242,9 +396,9 @@ __global__ void bfix_kernel(PopView<Cfg> V, Phys<typename Cfg::real> k, int a, i
     int r1[3] = {q[0], q[1], q[2]};
     r1[a] = b + sgn;
     R tang = R(0);
-    const int at[2] = {a1, a2};
+#pragma unroll
     for (int t = 0; t < 2; ++t) {
-        const int ax = at[t];
+        const int ax = t == 0 ? a1 : a2;
         if (n[ax] == 1) continue;
         int rp[3] = {r1[0], r1[1], r1[2]}, rm[3] = {r1[0], r1[1], r1[2]};
         rp[ax] = wrap_coord(r1[ax] + 1, n[ax], V.periodic[ax]);
@@ -264,10 +418,7 @@ __global__ void bfix_kernel(PopView<Cfg> V, Phys<typename Cfg::real> k, int a, i
     R fv[19], hv[8];
 #pragma unroll
     for (int i = 0; i < 19; ++i) fv[i] = ld_pop<Cfg>(V.fg + fg_elem(i, 0, cb, V.stride), V.hs.f[i]);
-    int hp = 0;  // the plane whose normal is axis a
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-        if (plane_normal(p) == a) hp = p;
+    constexpr int hp = plane_normal(0) == a ? 0 : (plane_normal(1) == a ? 1 : 2);  // the plane whose normal is axis a
 #pragma unroll
     for (int j = 0; j < 8; ++j) hv[j] = (R)V.h[h_elem(8 * hp + j, cb, V.stride)];
     const R dB = Bn_new - so.B[a];
@@ -339,8 +490,10 @@ __global__ void prim_component_kernel(PopView<Cfg> V, int P, typename Cfg::prim*
 }
 
 
+// Bound by the float64 rate like the initial state, not by memory (176 bytes a cell):
+// ~35 float64 instructions a cell, the conversions on the integer pipes.
 template <class Cfg>
-__global__ void moments_kernel(PopView<Cfg> V, Phys<double> k, double* out)
+__global__ void __launch_bounds__(128) moments_kernel(PopView<Cfg> V, Phys<double> k, double* out)
 {
     const int64_t N = (int64_t)V.nx * V.ny * V.nz;
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -349,20 +502,23 @@ __global__ void moments_kernel(PopView<Cfg> V, Phys<double> k, double* out)
     {
         typename Cfg::real pv[NPRIM];
         ld_prims<Cfg>(V.prim + prim_elem(0, c, V.stride), V.stride, pv);
-        s.n = (double)pv[P_N];
-        s.eps = (double)pv[P_EPS];
+        s.n = widen(pv[P_N]);
+        s.eps = widen(pv[P_EPS]);
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            s.u[a] = (double)pv[P_U + a];
-            s.E[a] = (double)pv[P_E + a];
-            s.B[a] = (double)pv[P_B + a];
+            s.u[a] = widen(pv[P_U + a]);
+            s.E[a] = widen(pv[P_E + a]);
+            s.B[a] = widen(pv[P_B + a]);
         }
-        s.rho = (double)pv[P_RHO];
+        s.rho = widen(pv[P_RHO]);
     }
+    const double g = rsqrt_newton(1.0 - (s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2]) * (k.inv_c * k.inv_c));
     double J[3];
-    ohm_current(s.E, s.u, s.B, s.rho, k, J);
+    ohm_current_g(s.E, s.u, s.B, s.rho, g, k, J);
     out[0 * N + c] = s.n;
     out[1 * N + c] = k.gm1 * (s.eps - s.n * k.c2);
     out[2 * N + c] = s.eps;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         out[(3 + a) * N + c] = s.u[a];
         out[(6 + a) * N + c] = s.E[a];
@@ -434,7 +590,6 @@ __global__ void diag_kernel(PopView<Cfg> V, Phys<double> k, RefState r, double* 
             bad = bad || !isfinite(hi);
             rho += hi;
         }
-#pragma unroll
         {
             R pv[NPRIM];
             ld_prims<Cfg>(V.prim + prim_elem(0, c, V.stride), V.stride, pv);
@@ -596,7 +751,7 @@ cudaError_t launch_init(const PopView<Cfg>& V, const InitInputs& in, const Phys<
                         cudaStream_t s)
 {
     const int64_t N = (int64_t)V.nx * V.ny * V.nz;
-    init_kernel<Cfg><<<blocks_for(N, 128), 128, 0, s>>>(V, in, k, bad);
+    init_kernel<Cfg><<<blocks_for(N, 128), 128, 0, s>>>(V, in, k, 1.0 / k.gm1, k.eps0 / (2.0 * k.dx), bad);
     return cudaGetLastError();
 }
 
@@ -625,11 +780,17 @@ cudaError_t launch_boundaries(const PopView<Cfg>& V, const Phys<typename Cfg::re
     for (int a = 0; a < 3; ++a) {
         const bool lo = bc[2 * a] != 0 && n[a] >= 3, hi = bc[2 * a + 1] != 0 && n[a] >= 3;
         const int64_t m = (int64_t)n[(a + 1) % 3] * n[(a + 2) % 3];
+        auto fix = [&](int64_t cells, int hi_first, int nfaces) {
+            const unsigned nb = blocks_for(cells, 128);
+            if (a == 0) bfix_kernel<Cfg, 0><<<nb, 128, 0, s>>>(V, k, hi_first, nfaces);
+            if (a == 1) bfix_kernel<Cfg, 1><<<nb, 128, 0, s>>>(V, k, hi_first, nfaces);
+            if (a == 2) bfix_kernel<Cfg, 2><<<nb, 128, 0, s>>>(V, k, hi_first, nfaces);
+        };
         if (lo && hi && n[a] >= 4) {
-            bfix_kernel<Cfg><<<blocks_for(2 * m, 128), 128, 0, s>>>(V, k, a, 0, 2);
+            fix(2 * m, 0, 2);
         } else {
-            if (lo) bfix_kernel<Cfg><<<blocks_for(m, 128), 128, 0, s>>>(V, k, a, 0, 1);
-            if (hi) bfix_kernel<Cfg><<<blocks_for(m, 128), 128, 0, s>>>(V, k, a, 1, 1);
+            if (lo) fix(m, 0, 1);
+            if (hi) fix(m, 1, 1);
         }
     }
     if (bc[4] == 2 && layers > 0 && drive_uv) {

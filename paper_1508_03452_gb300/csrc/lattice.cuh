@@ -103,6 +103,18 @@ __device__ __forceinline__ R sq(R a) { return a * a; }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return a * b; }
 
+// 1/sqrt(x), x >= 0, in float64: one third-order step r + r e (1/2 + 3/8 e), e = 1 - x r^2,
+// from the hardware's approximation (five FP64 instructions; rsqrt and the IEEE
+// square root and division take two to four times as many)
+__device__ __forceinline__ double rsqrt_newton(double x)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x * r, r, 1.0);
+    const double q = fma(r * e, fma(0.375, e, 0.5), r);
+    return ((unsigned)__double2hiint(r) & 0x7ff00000u) == 0x7ff00000u ? r : q;  // x = 0: infinity
+}
+
 __device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
 
@@ -280,6 +292,42 @@ __device__ __forceinline__ R k_aw(const EqCell<R>& q)
         return q.kf - R(c19(I, a)) * q.kq[a];
     } else {
         return q.kf - R(c19(I, a)) * q.kq[a] - R(c19(I, b)) * q.kq[b];
+    }
+}
+
+// Terms of the float64 equilibria, the direction weights taken in: f^eq of the
+// opposite directions +-c is E +- O with E even and O odd in c, and so is g^eq
+// (198 FP64 instructions per cell instead of 237 direction by direction).
+struct EqEven {
+    double f0, g0;                         // rest pair
+    double fe_ax[3], fo_ax[3], fe_dg[3], fo_dg[3], fx[3];
+    double ge_ax[3], go_ax[3], ge_dg[3], go_dg[3], gx[3];
+    double kf, kq[3];
+};
+__device__ __forceinline__ void eq_even(const EqCell<double>& q, EqEven& e)
+{
+    constexpr double wa = w19(1), wd = w19(7), va = wg19(1), vd = wg19(7);
+    e.f0 = mul_rn(w19(0), q.f_rest);
+    e.g0 = mul_rn(wg19(0), q.g_base);
+    double base[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        base[a] = q.g_base + q.g_sq[a];
+        e.fe_ax[a] = mul_rn(wa, q.f_even_ax[a]);
+        e.fo_ax[a] = mul_rn(wa, q.f_odd[a]);
+        e.fo_dg[a] = mul_rn(wd, q.f_odd[a]);
+        e.ge_ax[a] = mul_rn(va, base[a]);
+        e.go_ax[a] = mul_rn(va, q.g_lin[a]);
+        e.go_dg[a] = mul_rn(vd, q.g_lin[a]);
+        e.kq[a] = q.kq[a];
+    }
+    e.kf = q.kf;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        e.fe_dg[m] = mul_rn(wd, q.f_even_dg[m]);
+        e.fx[m] = mul_rn(wd, q.f_cross[m]);
+        e.ge_dg[m] = mul_rn(vd, (base[m == 2 ? 1 : 0] + q.g_sq[m == 0 ? 1 : 2]));
+        e.gx[m] = mul_rn(vd, q.g_x[m]);
     }
 }
 

@@ -541,42 +541,6 @@ __device__ __forceinline__ void collide_fg(const StepArgs<Cfg>& A, typename Cfg:
     }
 }
 
-// Terms of the float64 collision, the direction weights taken in: f^eq of the
-// opposite directions +-c is E +- O with E even and O odd in c, and so is g^eq
-// (198 FP64 instructions per cell instead of 237 direction by direction).
-struct EqEven {
-    double f0, g0;                         // rest pair
-    double fe_ax[3], fo_ax[3], fe_dg[3], fo_dg[3], fx[3];
-    double ge_ax[3], go_ax[3], ge_dg[3], go_dg[3], gx[3];
-    double kf, kq[3];
-};
-__device__ __forceinline__ void eq_even(const EqCell<double>& q, EqEven& e)
-{
-    constexpr double wa = w19(1), wd = w19(7), va = wg19(1), vd = wg19(7);
-    e.f0 = mul_rn(w19(0), q.f_rest);
-    e.g0 = mul_rn(wg19(0), q.g_base);
-    double base[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        base[a] = q.g_base + q.g_sq[a];
-        e.fe_ax[a] = mul_rn(wa, q.f_even_ax[a]);
-        e.fo_ax[a] = mul_rn(wa, q.f_odd[a]);
-        e.fo_dg[a] = mul_rn(wd, q.f_odd[a]);
-        e.ge_ax[a] = mul_rn(va, base[a]);
-        e.go_ax[a] = mul_rn(va, q.g_lin[a]);
-        e.go_dg[a] = mul_rn(vd, q.g_lin[a]);
-        e.kq[a] = q.kq[a];
-    }
-    e.kf = q.kf;
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {
-        e.fe_dg[m] = mul_rn(wd, q.f_even_dg[m]);
-        e.fx[m] = mul_rn(wd, q.f_cross[m]);
-        e.ge_dg[m] = mul_rn(vd, (base[m == 2 ? 1 : 0] + q.g_sq[m == 0 ? 1 : 2]));
-        e.gx[m] = mul_rn(vd, q.g_x[m]);
-    }
-}
-
 // post-collision f and g of group G (directions I = 2G - 1 and -I) from the streamed ones
 template <int G>
 __device__ __forceinline__ V4<double> collide_even(const EqEven& e, const V4<double>& d, double inv_tau)
