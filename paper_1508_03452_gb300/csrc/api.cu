@@ -1616,11 +1616,11 @@ int lbrmhd_set_mlp_weights(lbrmhd_handle h, const float* d_params)
     if (!h) return LBRMHD_ERR_BAD_ARG;
     if (!d_params) return fail(h, LBRMHD_ERR_BAD_ARG, "NULL parameters");
     LB_CK(cudaSetDevice(h->device));
-    if (!h->d_mlp && cudaMalloc(&h->d_mlp, lbrmhd_mlp_blob_bytes()) != cudaSuccess) {
+    if (!h->d_mlp && cudaMalloc(&h->d_mlp, lb::mlp_step_weight_bytes()) != cudaSuccess) {
         h->d_mlp = nullptr;
         return fail(h, LBRMHD_ERR_OOM, "network blob allocation failed");
     }
-    if (lb::launch_mlp_pack_warp(d_params, h->d_mlp, h->stream) != cudaSuccess)
+    if (lb::launch_mlp_pack_step(d_params, h->d_mlp, h->stream) != cudaSuccess)
         return fail(h, LBRMHD_ERR_CUDA, "packing the network failed");
     h->mlp_set = true;
     runs_changed(h);  // the kernel arguments carry the blob pointer

@@ -16,6 +16,7 @@
 
 #include "lbrmhd.h"
 #include "mlp.cuh"
+#include "mlp_tc.cuh"
 
 namespace lb {
 
@@ -327,38 +328,41 @@ __global__ void __launch_bounds__(32 * kReduceShares) mlp_reduce_kernel(const fl
     }
 }
 
-// float32 parameters -> bf16 inference blob in fragment order (zero padding)
-// (WARP: the step kernel's own copy, fragments in warp order)
-template <bool WARP>
+// float32 parameters -> bf16 inference blob in fragment order (zero padding); STEP:
+// the step kernels' own two copies instead, fragments in warp order (mma.sync), then
+// the tensor core's order (mlp_tc.cuh)
+template <bool STEP>
 __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __restrict__ blob)
 {
-    __nv_bfloat16* B = reinterpret_cast<__nv_bfloat16*>(blob);
-    struct Out {  // element e of the blob in its own order
-        __nv_bfloat16* p;
-        __device__ __nv_bfloat16& operator[](int e) const
-        {
-            return p[WARP ? 4 * mlp_warp_order(e / 4) + e % 4 : e];
+    __nv_bfloat16* W = reinterpret_cast<__nv_bfloat16*>(blob);
+    __nv_bfloat16* C = reinterpret_cast<__nv_bfloat16*>(blob + MLPD_BYTES);
+    float* bias = reinterpret_cast<float*>(blob + MLPD_NBF16 * 2);
+    // weight (r, k) of the layer that starts at `at` of the blob and `tc` of the tensor core's copy
+    auto put = [&](int at, int tc, int r, int k, int K, float v) {
+        const int e = at + mlpd_frag_index(r, k, K);
+        const __nv_bfloat16 b = __float2bfloat16_rn(v);
+        W[STEP ? 4 * mlp_warp_order(e / 4) + e % 4 : e] = b;
+        if constexpr (STEP) {
+            if (!(tc == MLPT_W1 && k >= MLP_IN && k < MLP_IN + 3))  // (the bias inputs)
+                C[tc + mlpt_index(r, k, tc == MLPT_W2 || tc == MLPT_W3 ? MLPT_KB : K)] = b;
         }
     };
-    const Out W{B};
-    float* bias = reinterpret_cast<float*>(blob + MLPD_NBF16 * 2);
     const int total = MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H + MLPD_NBIAS;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         // i enumerates (layer, r, k) in row-major order, then the biases
         if (i < MLP_H * MLP_K1) {
             const int r = i / MLP_K1, k = i % MLP_K1;
-            W[MLPD_W1 + mlpd_frag_index(r, k, MLP_K1)] =
-                __float2bfloat16_rn(k < MLP_IN ? P[MLP_W1 + r * MLP_IN + k] : 0.0f);
+            put(MLPD_W1, MLPT_W1, r, k, MLP_K1, k < MLP_IN ? P[MLP_W1 + r * MLP_IN + k] : 0.0f);
         } else if (i < MLP_H * MLP_K1 + MLP_H * MLP_H) {
             const int j = i - MLP_H * MLP_K1, r = j / MLP_H, k = j % MLP_H;
-            W[MLPD_W2 + mlpd_frag_index(r, k, MLP_H)] = __float2bfloat16_rn(P[MLP_W2 + r * MLP_H + k]);
+            put(MLPD_W2, MLPT_W2, r, k, MLP_H, P[MLP_W2 + r * MLP_H + k]);
         } else if (i < MLP_H * MLP_K1 + 2 * MLP_H * MLP_H) {
             const int j = i - MLP_H * MLP_K1 - MLP_H * MLP_H, r = j / MLP_H, k = j % MLP_H;
-            W[MLPD_W3 + mlpd_frag_index(r, k, MLP_H)] = __float2bfloat16_rn(P[MLP_W3 + r * MLP_H + k]);
+            put(MLPD_W3, MLPT_W3, r, k, MLP_H, P[MLP_W3 + r * MLP_H + k]);
         } else if (i < MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H) {
             const int j = i - MLP_H * MLP_K1 - 2 * MLP_H * MLP_H, r = j / MLP_H, k = j % MLP_H;
-            W[MLPD_W4 + mlpd_frag_index(r, k, MLP_H)] =
-                __float2bfloat16_rn(r < MLP_OUT ? P[MLP_W4 + r * MLP_H + k] : 0.0f);
+            put(MLPD_W4, MLPT_W4, r, k, MLP_H, r < MLP_OUT ? P[MLP_W4 + r * MLP_H + k] : 0.0f);
+            if constexpr (STEP) C[MLPT_W4 + mlpt_index(r + 8, k, MLP_H)] = __float2bfloat16_rn(0.0f);
         } else {
             const int j = i - (MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H);
             float val = 0.0f;
@@ -367,6 +371,12 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
             else if (j < 192) val = P[MLP_B3 + j - 128];
             else if (j < 192 + MLP_OUT) val = P[MLP_B4 + j - 192];
             bias[j] = val;
+            if constexpr (STEP) {
+                if (j < 3 * MLP_H)
+                    mlpt_put_bias(C, j / MLP_H, j % MLP_H, val);
+                else if (j < 3 * MLP_H + MLP_OUT)
+                    reinterpret_cast<float*>(blob + MLPD_BYTES + MLPT_BIAS)[j - 3 * MLP_H] = val;
+            }
         }
     }
 }
@@ -374,7 +384,7 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
 // Standalone inference: a warp takes 32 rows at a time through the network, the
 // activations staying in its registers from layer to layer (mlp_forward_frag),
 // the weights read from the block's shared copy; same products and sums in the
-// same order as the step kernel's. Bound by the warp-level tensor-core rate: 168
+// same order as the batched step kernels'. Bound by the warp-level tensor-core rate: 168
 // mma.sync per 32 rows, 16 clocks each on a scheduler's pipe, are 66 us for
 // 1,000,003 rows, which is what it takes. The rows arrive as coalesced 16-byte
 // loads for the next tile while this one is computed. Before, activations went
@@ -445,7 +455,9 @@ __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks) mlp_infer_kern
     }
 }
 
-cudaError_t launch_mlp_pack_warp(const float* params, unsigned char* blob, cudaStream_t s)
+int mlp_step_weight_bytes() { return MLPD_BYTES + MLPT_BYTES; }
+
+cudaError_t launch_mlp_pack_step(const float* params, unsigned char* blob, cudaStream_t s)
 {
     mlp_pack_kernel<true><<<32, 256, 0, s>>>(params, blob);
     return cudaGetLastError();

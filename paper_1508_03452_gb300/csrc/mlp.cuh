@@ -6,9 +6,12 @@
 // Parameters (float32 master copy, MLP_NPARAM values): W1[64][20] b1[64]
 // W2[64][64] b2[64] W3[64][64] b3[64] W4[4][64] b4[4], W[out][in].
 //
-// Inference inside the step kernel uses warp-level bf16 tensor-core MMA
-// (mma.sync m16n8k16, float32 accumulation): each warp owns the 32 cells (rows)
-// of its threads, so no block-wide barrier is needed.
+// Inference inside the tile, batched and persistent step kernels and the standalone one
+// use warp-level bf16 tensor-core MMA (mma.sync m16n8k16, float32 accumulation): each
+// warp owns the 32 cells (rows) of its threads, so no block-wide barrier is needed and no
+// block holds tensor memory while it waits for another. The one-run step kernel uses
+// the tensor-memory form (mlp_tc.cuh); there a result a rounding away only starts the
+// eigen-solve elsewhere, where the standalone inference's is the user's.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -202,7 +205,10 @@ __device__ __forceinline__ void mlp_forward_frag(const __nv_bfloat16* rows, cons
     }
 }
 
-// float32 parameters (device) -> blob with its fragments in warp order, on stream s
-cudaError_t launch_mlp_pack_warp(const float* params, unsigned char* blob, cudaStream_t s);
+// float32 parameters (device) -> the step kernels' copies of the weights
+// (mlp_step_weight_bytes() bytes), on stream s: the blob with its fragments in warp
+// order, then the tensor core's order
+int mlp_step_weight_bytes();
+cudaError_t launch_mlp_pack_step(const float* params, unsigned char* blob, cudaStream_t s);
 
 }  // namespace lb

@@ -20,6 +20,7 @@
 #pragma once
 #include "common.cuh"
 #include "mlp.cuh"
+#include "mlp_tc.cuh"
 #include "tma.cuh"
 
 namespace lb {
@@ -953,6 +954,13 @@ struct TileStages<kTileStages, Cfg> {
     }
 };
 
+// The block's tensor-memory network (mlp_tc.cuh) in the one-run step kernel
+struct TcCtx {
+    const unsigned char* w;  // weights in shared memory, arriving on bar[0]
+    uint64_t* bar;           // [0] the weights, [1] the products
+    uint32_t tmem;           // the block's columns, given back after the network
+};
+
 // One cell update (x, y, z) of one run; `tid` is the thread's index in its
 // block of kStepThreads threads (its rows of the shared-memory buffers). Threads of
 // cells outside the grid return at once, except in the learned-seed variant,
@@ -961,9 +969,12 @@ struct TileStages<kTileStages, Cfg> {
 // TILE: a cell of an interior tile of the TMA tile path (2-D, periodic,
 // every cell active): its inputs come from the block's ring and primitive
 // buffers (tc), its outputs go to the block's shared-memory output tiles.
-template <class Cfg, bool IS3D, int SEED, bool OPEN, bool TILE = false, int NTH = kStepThreads>
+// TC: the learned seed's network runs block-wide in tensor memory (*tm), every
+// thread of the block calling; otherwise warp by warp.
+template <class Cfg, bool IS3D, int SEED, bool OPEN, bool TILE = false, int NTH = kStepThreads, bool TC = false>
 __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, const int z, const int tid,
-                                          unsigned char* smem_raw, const TileCtx<Cfg>* tc = nullptr)
+                                          unsigned char* smem_raw, const TileCtx<Cfg>* tc = nullptr,
+                                          const TcCtx* tm = nullptr)
 {
     constexpr int nth = NTH;  // threads of the block: a compile-time stride of the shared-memory slots
     using R = typename Cfg::real;
@@ -1093,31 +1104,49 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
         mlp_features(k.eps_r + T[0][0], T0a, Tab, k.n_r + dN0, Nq, old.E, old.B, feat);
     }
     if constexpr (SEED == SEED_MLP) {
-        __nv_bfloat16* act =
-            reinterpret_cast<__nv_bfloat16*>(smem_raw + (size_t)kStepSlots * sizeof(R) * nth);
-        __nv_bfloat16* row = act + tid * MLP_FROW;
+        float out_f[MLP_OUT];
+        if constexpr (TC) {
+            uint32_t xb[MLP_IN / 2];
 #pragma unroll
-        for (int j = 0; j < 32; j += 2)
-            *reinterpret_cast<__nv_bfloat162*>(row + j) =
-                __floats2bfloat162_rn(j < MLP_IN ? feat[j] : 0.0f, j + 1 < MLP_IN ? feat[j + 1] : 0.0f);
-        __syncwarp();
-        const int lane = tid & 31;
+            for (int j = 0; j < MLP_IN / 2; ++j) xb[j] = pack_bf16(feat[2 * j], feat[2 * j + 1]);
+            const bool in = mbar_wait_bounded(&tm->bar[0], 0u);
+            __syncwarp();
+            uint32_t phase = 0;
+            const bool got = mlp_forward_tc(xb, tm->w, tm->tmem, &tm->bar[1], phase, tid, out_f, in);
+            if (tid < 32) tc_dealloc(tm->tmem);
+            if (!got) {  // a wait ran out: the eigen-solve starts from the previous velocity
+                if (tid == 0) atomicOr(A.status, STATUS_TMA_TIMEOUT);
 #pragma unroll
-        for (int part = 0; part < 2 / kMlpTiles; ++part) {
-            __nv_bfloat16* rows = act + ((tid & ~31) + 16 * kMlpTiles * part) * MLP_FROW;
-            float y[kMlpTiles][4];
-            mlp_forward_frag<kMlpTiles, true>(rows, A.mlp, y);
-            __syncwarp();  // the feature rows have been read: the outputs take their place
-            if ((lane & 3) < 2)
+                for (int a = 0; a < 3; ++a) out_f[a] = (float)(old.u[a] * k.inv_c);
+            }
+        } else {
+            __nv_bfloat16* act =
+                reinterpret_cast<__nv_bfloat16*>(smem_raw + (size_t)kStepSlots * sizeof(R) * nth);
+            __nv_bfloat16* row = act + tid * MLP_FROW;
 #pragma unroll
-                for (int mt = 0; mt < kMlpTiles; ++mt)
+            for (int j = 0; j < 32; j += 2)
+                *reinterpret_cast<__nv_bfloat162*>(row + j) =
+                    __floats2bfloat162_rn(j < MLP_IN ? feat[j] : 0.0f, j + 1 < MLP_IN ? feat[j + 1] : 0.0f);
+            __syncwarp();
+            const int lane = tid & 31;
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh)
-                        *reinterpret_cast<float2*>(rows + (16 * mt + (lane >> 2) + 8 * hh) * MLP_FROW + 4 * (lane & 3)) =
-                            make_float2(y[mt][2 * hh], y[mt][2 * hh + 1]);
+            for (int part = 0; part < 2 / kMlpTiles; ++part) {
+                __nv_bfloat16* rows = act + ((tid & ~31) + 16 * kMlpTiles * part) * MLP_FROW;
+                float y[kMlpTiles][4];
+                mlp_forward_frag<kMlpTiles, true>(rows, A.mlp, y);
+                __syncwarp();  // the feature rows have been read: the outputs take their place
+                if ((lane & 3) < 2)
+#pragma unroll
+                    for (int mt = 0; mt < kMlpTiles; ++mt)
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh)
+                            *reinterpret_cast<float2*>(rows + (16 * mt + (lane >> 2) + 8 * hh) * MLP_FROW + 4 * (lane & 3)) =
+                                make_float2(y[mt][2 * hh], y[mt][2 * hh + 1]);
+            }
+            __syncwarp();
+            const float* out = reinterpret_cast<const float*>(row);
+            out_f[0] = out[0], out_f[1] = out[1], out_f[2] = out[2];
         }
-        __syncwarp();
-        const float* out_f = reinterpret_cast<const float*>(row);
         R sb[3] = {(R)out_f[0], (R)out_f[1], (R)out_f[2]};
         const R sb2 = sb[0] * sb[0] + sb[1] * sb[1] + sb[2] * sb[2];
         const R lim = R(0.9);  // keep the guess well inside the light cone
@@ -1398,7 +1427,32 @@ __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::
     const int z = IS3D && back ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = by * blockDim.y + threadIdx.y;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-    step_cell<Cfg, IS3D, SEED, OPEN>(A, x, y, z, tid, smem_raw);
+    if constexpr (SEED == SEED_MLP) {
+        // tensor memory (128 of 512 columns a block, three blocks an SM at most) and, in
+        // flight while the block streams, the network's weights
+        constexpr size_t slots = (size_t)kStepSlots * sizeof(typename Cfg::real) * kStepThreads;
+        static_assert(slots % 16 == 0 && kStepThreads == kTcRows, "one row of the network per thread");
+        TcCtx tm;
+        tm.w = smem_raw + slots;
+        tm.bar = reinterpret_cast<uint64_t*>(smem_raw + slots + MLPT_BYTES);
+        uint32_t* tmem_sh = reinterpret_cast<uint32_t*>(tm.bar + 2);
+        if (tid == 0) {
+            mbar_init(&tm.bar[0], 1u);
+            mbar_init(&tm.bar[1], 1u);
+            mbar_init_fence();
+            mbar_arrive_expect_tx(&tm.bar[0], MLPT_BYTES);
+            bulk_load(smem_raw + slots, A.mlp + MLPD_BYTES, MLPT_BYTES, &tm.bar[0]);
+        }
+        if (tid < 32) tc_alloc(tmem_sh);
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        tm.tmem = *tmem_sh;
+        mlp_tc_constants(tm.tmem, tid);
+        step_cell<Cfg, IS3D, SEED, OPEN, false, kStepThreads, true>(A, x, y, z, tid, smem_raw, nullptr, &tm);
+    } else {
+        step_cell<Cfg, IS3D, SEED, OPEN>(A, x, y, z, tid, smem_raw);
+    }
 }
 
 template <class Cfg, int NTH = kStepThreads>
@@ -1609,7 +1663,7 @@ __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::
 template <class Cfg>
 size_t step_smem_bytes(int seed)
 {
-    return step_cell_smem<Cfg>(seed);
+    return seed == SEED_MLP ? step_cell_smem<Cfg>(SEED_PREV) + MLPT_BYTES + 3 * sizeof(uint64_t) : step_cell_smem<Cfg>(seed);
 }
 
 template <class Cfg>
