@@ -298,18 +298,21 @@ __device__ __forceinline__ R k_aw(const EqCell<R>& q)
 // Terms of the float64 equilibria, the direction weights taken in: f^eq of the
 // opposite directions +-c is E +- O with E even and O odd in c, and so is g^eq
 // (198 FP64 instructions per cell instead of 237 direction by direction).
-struct EqEven {
-    double f0, g0;                         // rest pair
-    double fe_ax[3], fo_ax[3], fe_dg[3], fo_dg[3], fx[3];
-    double ge_ax[3], go_ax[3], ge_dg[3], go_dg[3], gx[3];
-    double kf, kq[3];
+template <class R>
+struct EqEvenT {
+    R f0, g0;                         // rest pair
+    R fe_ax[3], fo_ax[3], fe_dg[3], fo_dg[3], fx[3];
+    R ge_ax[3], go_ax[3], ge_dg[3], go_dg[3], gx[3];
+    R kf, kq[3];
 };
-__device__ __forceinline__ void eq_even(const EqCell<double>& q, EqEven& e)
+using EqEven = EqEvenT<double>;
+template <class R>
+__device__ __forceinline__ void eq_even(const EqCell<R>& q, EqEvenT<R>& e)
 {
-    constexpr double wa = w19(1), wd = w19(7), va = wg19(1), vd = wg19(7);
-    e.f0 = mul_rn(w19(0), q.f_rest);
-    e.g0 = mul_rn(wg19(0), q.g_base);
-    double base[3];
+    const R wa(w19(1)), wd(w19(7)), va(wg19(1)), vd(wg19(7));
+    e.f0 = mul_rn(R(w19(0)), q.f_rest);
+    e.g0 = mul_rn(R(wg19(0)), q.g_base);
+    R base[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         base[a] = q.g_base + q.g_sq[a];
