@@ -17,6 +17,7 @@
 #include "lbrmhd.h"
 #include "mlp.cuh"
 #include "mlp_tc.cuh"
+#include "tma.cuh"
 
 namespace lb {
 
@@ -44,11 +45,6 @@ __host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t x)
     x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
     return x ^ (x >> 31);
 }
-
-// the grid's predecessor on the stream has finished and its writes are visible
-// (a programmatic launch may start earlier); let the successor's blocks launch
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // 16 bytes from global memory (through L2) into shared memory, and the wait for
 // all of a thread's copies
@@ -384,10 +380,9 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
 // Standalone inference: a warp takes 32 rows at a time through the network, the
 // activations staying in its registers from layer to layer (mlp_forward_frag),
 // the weights read from the block's shared copy; same products and sums in the
-// same order as the batched step kernels'. Bound by the warp-level tensor-core rate: 168
-// mma.sync per 32 rows, 16 clocks each on a scheduler's pipe, are 66 us for
-// 1,000,003 rows, which is what it takes. The rows arrive as coalesced 16-byte
-// loads for the next tile while this one is computed. Before, activations went
+// same order as the batched step kernels'. Bound by the warp-level matrix instructions
+// (168 mma.sync per 32 rows): 55 us for 1,000,003 rows. The rows arrive as coalesced
+// 16-byte loads for the next tile while this one is computed. Before, activations went
 // through shared memory, and the rows and the weight fragments were loaded at
 // strides: L1 92 % busy, 121 us.
 constexpr int kInferWarps = 4, kInferBlocks = 3;  // warps per block, blocks per SM (4: 128 registers spill, 74 us)
@@ -399,8 +394,19 @@ __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks) mlp_infer_kern
     __shared__ __align__(16) __nv_bfloat16 rows[kInferWarps][32 * MLP_FROW];
     const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
     // the blob's fragments (8 bytes a lane), those of a warp's lanes side by side
-    for (int i = threadIdx.x; i < MLPD_NBF16 / 4; i += 32 * kInferWarps)
-        reinterpret_cast<uint2*>(wts)[mlp_warp_order(i)] = __ldg(reinterpret_cast<const uint2*>(blob) + i);
+    // (unrolled, all loads in flight at once: a call of few rows is mostly this, 100 to
+    // 10,000 rows 3.3 us where the first kernel took 5.4)
+    constexpr int kFrags = MLPD_NBF16 / 4, kInferThreads = 32 * kInferWarps;
+    static_assert(kFrags % kInferThreads == 0 && MLPD_W2 / 4 % kInferThreads == 0 && MLPD_W3 / 4 % kInferThreads == 0 &&
+                      MLPD_W4 / 4 % kInferThreads == 0,
+                  "a pass of the threads stays in one layer");
+    uint2 frag[kFrags / kInferThreads];
+#pragma unroll
+    for (int j = 0; j < kFrags / kInferThreads; ++j)
+        frag[j] = __ldg(reinterpret_cast<const uint2*>(blob) + threadIdx.x + j * kInferThreads);
+#pragma unroll
+    for (int j = 0; j < kFrags / kInferThreads; ++j)
+        reinterpret_cast<uint2*>(wts)[mlp_warp_order(threadIdx.x, j * kInferThreads)] = frag[j];
     for (int i = threadIdx.x; i < MLPD_NBIAS; i += 32 * kInferWarps)
         reinterpret_cast<float*>(wts + MLPD_NBF16 * 2)[i] = __ldg(reinterpret_cast<const float*>(blob + MLPD_NBF16 * 2) + i);
     __nv_bfloat16* mine = rows[w];

@@ -91,14 +91,17 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint
 // that use them together, for two k-tiles at a time, are consecutive: a warp's
 // load is 512 bytes in a row. In the blob's own order the 8 rows of a fragment
 // lie K * 2 bytes apart, in the same shared-memory banks.
-__device__ __forceinline__ int mlp_warp_order(int i)
+// (i = base + at; a constant `at` that is the same side of the layers' starts for every
+// `base` settles the layer at compile time)
+__device__ __forceinline__ int mlp_warp_order(int base, int at)
 {
-    const int first = i < MLPD_W2 / 4 ? 0 : (i < MLPD_W3 / 4 ? MLPD_W2 / 4 : (i < MLPD_W4 / 4 ? MLPD_W3 / 4 : MLPD_W4 / 4));
+    const int first = at < MLPD_W2 / 4 ? 0 : (at < MLPD_W3 / 4 ? MLPD_W2 / 4 : (at < MLPD_W4 / 4 ? MLPD_W3 / 4 : MLPD_W4 / 4));
     const int kt_count = first == 0 ? MLP_K1 / 16 : MLP_H / 16;
-    const int j = i - first, t = j % 4, kt = (j / 4) % kt_count, r = j / (4 * kt_count);
+    const int j = base + (at - first), t = j % 4, kt = (j / 4) % kt_count, r = j / (4 * kt_count);
     const int lane = (r % 8) * 4 + t;
     return first + ((r / 8) * kt_count + (kt & ~1)) * 32 + 2 * lane + (kt & 1);
 }
+__device__ __forceinline__ int mlp_warp_order(int i) { return mlp_warp_order(0, i); }
 
 // a vector of the blob, in global memory (read-only path) or the block's shared copy
 template <bool GLOBAL, class T>

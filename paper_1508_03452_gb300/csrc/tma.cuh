@@ -87,6 +87,11 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+// the grid's predecessor on the stream has finished and its writes are visible
+// (a programmatic launch may start earlier); let the successor's blocks launch
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
