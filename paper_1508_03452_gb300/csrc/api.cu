@@ -542,7 +542,7 @@ int prepare_batch(lbrmhd_handle h, const lbrmhd_schedule& sc)
 // runs), issued on stream `s`; the host state (cur, step counters) is not
 // touched, so a caller can also issue a dry step whose output is discarded
 template <class Cfg>
-int issue_step(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, cudaStream_t s)
+int issue_step(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, cudaStream_t s, bool overlap)
 {
     using R = typename Cfg::real;
     const int out = 1 - in;
@@ -561,7 +561,7 @@ int issue_step(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, cudaStream_t 
         for (size_t ri = 0; ri < h->runs.size(); ++ri) {
             lb::TileLaunch tl{};
             const bool t = tile_launch<Cfg>(h, ri, in, &tl);
-            LB_CK(lb::launch_step<Cfg>(make_args<Cfg>(h, h->runs[ri], in), s, t ? &tl : nullptr));
+            LB_CK(lb::launch_step<Cfg>(make_args<Cfg>(h, h->runs[ri], in), s, t ? &tl : nullptr, overlap));
         }
     }
     for (const auto& r : h->runs) {
@@ -635,9 +635,15 @@ int issue_steps(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, int64_t n, c
     using R = typename Cfg::real;
     if (sc.kind == LBRMHD_SCHED_PERSISTENT) return issue_persistent<Cfg>(h, sc, in, n, s);
     const int S = sc.kind == LBRMHD_SCHED_PER_RUN ? std::min<int>(sc.streams, (int)h->runs.size()) : 1;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    bool overlap = s == h->cap_stream;  // (our own graphs; not a caller's)
+    if (!overlap) {
+        overlap = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+        if (!overlap) cudaGetLastError();
+    }
     if (S <= 1) {
         for (int64_t t = 0; t < n; ++t) {
-            const int rc = issue_step<Cfg>(h, sc, (int)((in + t) & 1), s);
+            const int rc = issue_step<Cfg>(h, sc, (int)((in + t) & 1), s, overlap);
             if (rc) return rc;
         }
         return LBRMHD_OK;
@@ -653,7 +659,7 @@ int issue_steps(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, int64_t n, c
             cudaStream_t st = h->aux[ri % S];
             lb::TileLaunch tl{};
             const bool t = tile_launch<Cfg>(h, ri, cin, &tl);
-            LB_CK(lb::launch_step<Cfg>(make_args<Cfg>(h, r, cin), st, t ? &tl : nullptr));
+            LB_CK(lb::launch_step<Cfg>(make_args<Cfg>(h, r, cin), st, t ? &tl : nullptr, overlap));
             if (has_open(r))
                 LB_CK(lb::launch_boundaries<Cfg>(view<Cfg>(r, 1 - cin), make_phys<R>(r.p, r.ref, runref(r)), r.p.bc,
                                                  r.p.drive_layers, r.d_drive, st));
@@ -1063,7 +1069,7 @@ int relax_run(lbrmhd_handle h, RunState& r, int max_iters, double tol, int* iter
         A.relax_in = h->d_io;
         A.relax_e = e;
         A.relax_red = h->d_small;
-        if (ce == cudaSuccess) ce = lb::launch_step<Cfg>(A, h->stream, nullptr);
+        if (ce == cudaSuccess) ce = lb::launch_step<Cfg>(A, h->stream, nullptr, false);
         if (ce == cudaSuccess && has_open(r))
             ce = lb::launch_boundaries<Cfg>(view<Cfg>(r, 1 - r.cur), make_phys<R>(r.p, r.ref, runref(r)), r.p.bc,
                                             r.p.drive_layers, r.d_drive, h->stream);
