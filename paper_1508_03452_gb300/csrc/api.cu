@@ -567,7 +567,7 @@ int issue_step(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, cudaStream_t 
     for (const auto& r : h->runs) {
         if (has_open(r))
             LB_CK(lb::launch_boundaries<Cfg>(view<Cfg>(r, out), make_phys<R>(r.p, r.ref, runref(r)), r.p.bc,
-                                             r.p.drive_layers, r.d_drive, s));
+                                             r.p.drive_layers, r.d_drive, overlap, s));
         if (capped(r)) LB_CK(lb::launch_umax_roll(r.d_umax, s));
     }
     return LBRMHD_OK;
@@ -662,7 +662,7 @@ int issue_steps(lbrmhd_handle h, const lbrmhd_schedule& sc, int in, int64_t n, c
             LB_CK(lb::launch_step<Cfg>(make_args<Cfg>(h, r, cin), st, t ? &tl : nullptr, overlap));
             if (has_open(r))
                 LB_CK(lb::launch_boundaries<Cfg>(view<Cfg>(r, 1 - cin), make_phys<R>(r.p, r.ref, runref(r)), r.p.bc,
-                                                 r.p.drive_layers, r.d_drive, st));
+                                                 r.p.drive_layers, r.d_drive, overlap, st));
             if (capped(r)) LB_CK(lb::launch_umax_roll(r.d_umax, st));
         }
     }
@@ -1072,7 +1072,7 @@ int relax_run(lbrmhd_handle h, RunState& r, int max_iters, double tol, int* iter
         if (ce == cudaSuccess) ce = lb::launch_step<Cfg>(A, h->stream, nullptr, false);
         if (ce == cudaSuccess && has_open(r))
             ce = lb::launch_boundaries<Cfg>(view<Cfg>(r, 1 - r.cur), make_phys<R>(r.p, r.ref, runref(r)), r.p.bc,
-                                            r.p.drive_layers, r.d_drive, h->stream);
+                                            r.p.drive_layers, r.d_drive, false, h->stream);
         r.cur ^= 1;
         double red[2] = {0.0, 0.0};
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(red, h->d_small, sizeof(red), cudaMemcpyDeviceToHost, h->stream);

@@ -427,6 +427,7 @@ struct FixF<19, Cfg, R, DIFF> {
 template <class Cfg, int a>
 __global__ void __launch_bounds__(128) bfix_kernel(PopView<Cfg> V, Phys<typename Cfg::real> k, int hi_first, int nfaces)
 {
+    grid_wait();  // (a programmatic launch: see the step kernel)
     using R = typename Cfg::real;
     const int n[3] = {V.nx, V.ny, V.nz};
     constexpr int a1 = (a + 1) % 3, a2 = (a + 2) % 3;
@@ -511,6 +512,9 @@ __global__ void __launch_bounds__(128) bfix_kernel(PopView<Cfg> V, Phys<typename
         eq_cell(sn, k, qn);
         FixF<0, Cfg, R>::run(V, cb, qo, qn, fv);
     }
+    // at the end: what launches next reads the lines that this kernel's blocks share, so
+    // its launch has to come after every block's loads
+    grid_release();
 }
 
 // ---------------------------------------------------------------------------
@@ -850,19 +854,28 @@ cudaError_t launch_drive_profile(int nx, int ny, double u0, double* uv, cudaStre
 
 template <class Cfg>
 cudaError_t launch_boundaries(const PopView<Cfg>& V, const Phys<typename Cfg::real>& k, const int* bc, int layers,
-                              const double* drive_uv, cudaStream_t s)
+                              const double* drive_uv, bool overlap, cudaStream_t s)
 {
     const int n[3] = {V.nx, V.ny, V.nz};
+    cudaError_t err = cudaSuccess;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap ? 1 : 0;
     // (the copy of the interior neighbour into the open faces is done by the
     // step kernel itself; here the normal-B fix and the driving follow it)
     for (int a = 0; a < 3; ++a) {
         const bool lo = bc[2 * a] != 0 && n[a] >= 3, hi = bc[2 * a + 1] != 0 && n[a] >= 3;
         const int64_t m = (int64_t)n[(a + 1) % 3] * n[(a + 2) % 3];
         auto fix = [&](int64_t cells, int hi_first, int nfaces) {
-            const unsigned nb = blocks_for(cells, 128);
-            if (a == 0) bfix_kernel<Cfg, 0><<<nb, 128, 0, s>>>(V, k, hi_first, nfaces);
-            if (a == 1) bfix_kernel<Cfg, 1><<<nb, 128, 0, s>>>(V, k, hi_first, nfaces);
-            if (a == 2) bfix_kernel<Cfg, 2><<<nb, 128, 0, s>>>(V, k, hi_first, nfaces);
+            cfg.gridDim = dim3(blocks_for(cells, 128));
+            const cudaError_t e = cudaLaunchKernelEx(
+                &cfg, a == 0 ? bfix_kernel<Cfg, 0> : (a == 1 ? bfix_kernel<Cfg, 1> : bfix_kernel<Cfg, 2>), V, k, hi_first, nfaces);
+            if (err == cudaSuccess) err = e;
         };
         if (lo && hi && n[a] >= 4) {
             fix(2 * m, 0, 2);
@@ -875,7 +888,8 @@ cudaError_t launch_boundaries(const PopView<Cfg>& V, const Phys<typename Cfg::re
         const int nl = layers < V.nz ? layers : V.nz;
         drive_kernel<Cfg><<<blocks_for((int64_t)V.nx * V.ny * nl, 128), 128, 0, s>>>(V, k, nl, drive_uv);
     }
-    return cudaGetLastError();
+    const cudaError_t last = cudaGetLastError();
+    return err != cudaSuccess ? err : last;
 }
 
 template <class Cfg>
@@ -998,7 +1012,7 @@ cudaError_t launch_relax_history(const PopView<Cfg>& V, double* e, cudaStream_t 
     template cudaError_t launch_init<CFG>(const PopView<CFG>&, const InitInputs&, const Phys<double>&, int*,      \
                                           cudaStream_t);                                                           \
     template cudaError_t launch_boundaries<CFG>(const PopView<CFG>&, const Phys<CFG::real>&, const int*, int,      \
-                                                const double*, cudaStream_t);                                      \
+                                                const double*, bool, cudaStream_t);                                      \
     template cudaError_t launch_moments<CFG>(const PopView<CFG>&, const Phys<double>&, double*, cudaStream_t);     \
     template cudaError_t launch_prim_component<CFG>(const PopView<CFG>&, int, CFG::prim*, cudaStream_t);           \
     template cudaError_t launch_populations<CFG>(const PopView<CFG>&, const RefPops&, double*, double*, double*,  \

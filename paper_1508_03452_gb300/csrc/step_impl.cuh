@@ -693,16 +693,22 @@ constexpr int kStepSlots = 63;  // 19 f + 19 g + 25 h pre-collision values per c
 #define LB_STEP_BX 128  // block width along x (the block is LB_STEP_BX x 128 / LB_STEP_BX)
 #endif
 #ifndef LB_STEP_MIN_BLOCKS_F16
-#define LB_STEP_MIN_BLOCKS_F16 4  // float16-deviation storage: 128 registers (no spills) beat 96 by 12 %
+// float16-deviation storage, 2-D: 5 blocks (102 registers) against 4 of 128, 10 steps and
+// a read-out of 2048^2 4.90 -> 4.81 ms (with more instructions in the stencil 4 won)
+#define LB_STEP_MIN_BLOCKS_F16 5
+#endif
+#ifndef LB_STEP_MIN_BLOCKS_F16_3D
+#define LB_STEP_MIN_BLOCKS_F16_3D 4
 #endif
 #ifndef LB_STEP_MIN_BLOCKS_MLP
-#define LB_STEP_MIN_BLOCKS_MLP 3  // the learned-seed variant: 3 blocks (168 registers) beat 4 by 18 %
+#define LB_STEP_MIN_BLOCKS_MLP 3  // the learned-seed variant: 3 blocks (168 registers) beat 4 by 1 %, 2 by 23 %
 #endif
 // float64: 2 blocks
 template <class Cfg, int SEED, bool IS3D = false>
 struct StepMinBlocks {
     static constexpr int value = sizeof(typename Cfg::real) == 8 ? 2
                                  : SEED == SEED_MLP             ? LB_STEP_MIN_BLOCKS_MLP
+                                 : Cfg::kHalf && IS3D           ? LB_STEP_MIN_BLOCKS_F16_3D
                                  : Cfg::kHalf                   ? LB_STEP_MIN_BLOCKS_F16
                                  : IS3D                         ? LB_STEP_MIN_BLOCKS_3D
                                                                 : LB_STEP_MIN_BLOCKS;
@@ -1414,8 +1420,9 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
 
 // A programmatic launch (launch_step) may start while the kernel before it on the
 // stream drains; grid_wait returns when that has finished. grid_release comes after it:
-// when the next step's blocks launch, no kernel runs that reads their input buffer (the
-// step before last did), so no L1 line of it outlives their launch.
+// when the next kernel's blocks launch, none runs that reads the buffer they read (the step
+// before last did; the boundary kernels release at their end), so no L1 line of it
+// outlives their launch.
 // one run: a 2-D grid of blocks over (x, y) and z
 template <class Cfg, bool IS3D, int SEED, bool OPEN>
 __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::value)
@@ -1869,10 +1876,9 @@ struct LaunchRun {
     template <bool D, int S, bool O>
     cudaError_t run()
     {
-        // Steps of runs without open faces follow one another with nothing between, so they
-        // launch programmatically (64^2 cells, 8.3 -> 6.6 us a step; 1024^2 runs 1 %). Open
-        // runs have the boundary kernels between, which read and write the step's input in
-        // place.
+        // programmatic: 64^2 cells, 8.3 -> 6.6 us a step; 1024^2 runs 1 %; with
+        // the boundary kernel between, 512^2 1.08 -> 1.07 ms for 20 steps, the float64 line of
+        // 100 cells 30.4 -> 28.7 ms for 377
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = grid;
         cfg.blockDim = block;
@@ -1882,7 +1888,7 @@ struct LaunchRun {
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = overlap && !O ? 1 : 0;
+        cfg.numAttrs = overlap ? 1 : 0;
         return cudaLaunchKernelEx(&cfg, step_kernel<Cfg, D, S, O>, *A);
     }
 };
