@@ -1431,13 +1431,13 @@ __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_wait();
     grid_release();
-    // every second step (the input buffer of the upper address) walks the rows and
-    // layers backwards, so that it starts with what the step before wrote last and L2
-    // still holds: 97 x 61 x 75 cells 1.96 -> 1.90 ms for 20 steps, 512^2 1.15 -> 1.11;
-    // runs far larger than L2 (1024^2 and up) within 0.3 %
-    const bool back = reinterpret_cast<uintptr_t>(A.fgin) > reinterpret_cast<uintptr_t>(A.fgout);
+    // 2-D: every second step (the input buffer of the upper address) walks the rows
+    // backwards, so that it starts with what the step before wrote last and L2 still
+    // holds: 512^2 1.15 -> 1.11 ms for 20 steps; runs far larger than L2 (1024^2 and up)
+    // within 0.3 %. In 3-D the registers cost more (97 x 61 x 75 1.90 against 1.89 ms).
+    const bool back = !IS3D && reinterpret_cast<uintptr_t>(A.fgin) > reinterpret_cast<uintptr_t>(A.fgout);
     const int by = back ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
-    const int z = IS3D && back ? gridDim.z - 1 - blockIdx.z : blockIdx.z;
+    const int z = blockIdx.z;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = by * blockDim.y + threadIdx.y;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     if constexpr (SEED == SEED_MLP) {
