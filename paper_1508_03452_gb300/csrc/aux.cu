@@ -512,8 +512,6 @@ __global__ void __launch_bounds__(128) bfix_kernel(PopView<Cfg> V, Phys<typename
         eq_cell(sn, k, qn);
         FixF<0, Cfg, R>::run(V, cb, qo, qn, fv);
     }
-    // at the end: what launches next reads the lines that this kernel's blocks share, so
-    // its launch has to come after every block's loads
     grid_release();
 }
 

@@ -101,12 +101,14 @@ struct StepArgs {
     using hpop = typename Cfg::hpop;
     using prim = typename Cfg::prim;
     using real = typename Cfg::real;
-    const pop* __restrict__ fgin;  // f and g in the group order of fg_elem
-    const hpop* __restrict__ hin;  // h in the pair order of h_elem
-    const prim* __restrict__ pin;
-    pop* __restrict__ fgout;
-    hpop* __restrict__ hout;
-    prim* __restrict__ pout;
+    // (not __restrict__: a programmatic launch's predecessor, and the step before in a
+    // persistent launch, write the input buffers while the kernel lives)
+    const pop* fgin;  // f and g in the group order of fg_elem
+    const hpop* hin;  // h in the pair order of h_elem
+    const prim* pin;
+    pop* fgout;
+    hpop* hout;
+    prim* pout;
     int nx, ny, nz;
     int64_t stride;  // elements between consecutive planes
     int periodic[3];
@@ -143,14 +145,53 @@ constexpr int STATUS_BARRIER_TIMEOUT = 2;  // a persistent launch's grid barrier
 // open_mask bit for runs that need the open-variant code without an open face
 constexpr int OPEN_EXTRA = 8;
 
+// Loads of a run's state. A kernel that is launched while its predecessor drains, or
+// that makes several steps, lives while these buffers are written, so they are ordinary
+// loads, which the memory model orders after the wait for the writer; the read-only
+// path (__ldg, __restrict__) is for data that nobody writes while a kernel lives.
+// ORDERED (the float16 step kernels): loads the compiler keeps in program order. Free to
+// move them across the stores of the shared-memory slots it holds more of a cell in
+// registers than float16's 96 allow (256 bytes of spills; 2048^2, 10 steps and a
+// read-out, 6.9 ms against 4.8). Float32 gains from the freedom, against the read-only
+// path (64^2 cells 658 -> 628 us, 97 x 61 x 75 1.86 -> 1.81 ms, 30,000 cells in 3-D 151
+// -> 146 us, 1024^2 runs as fast; open 2-D runs of 200 x 100 cells 2 % slower). Only
+// where a step never writes what it reads: the compiler may move a store before such a
+// load (but not across the persistent launch's barrier between two steps).
+template <bool ORDERED, class T>
+__device__ __forceinline__ T ld_state(const T* p)
+{
+    if constexpr (!ORDERED) {
+        return *p;
+    } else if constexpr (sizeof(T) == 4) {
+        unsigned u;
+        asm volatile("ld.global.u32 %0, [%1];" : "=r"(u) : "l"(p));
+        T v;
+        memcpy(&v, &u, sizeof(v));
+        return v;
+    } else if constexpr (sizeof(T) == 8) {
+        uint2 u;
+        asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(p));
+        T v;
+        memcpy(&v, &u, sizeof(v));
+        return v;
+    } else {
+        static_assert(sizeof(T) == 16, "the vectors of a float16 run");
+        uint4 u;
+        asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w) : "l"(p));
+        T v;
+        memcpy(&v, &u, sizeof(v));
+        return v;
+    }
+}
+
 // population load / store in the configured format
 template <class Cfg>
 __device__ __forceinline__ typename Cfg::real ld_pop(const typename Cfg::pop* p, float scale)
 {
     if constexpr (Cfg::kHalf)
-        return __half2float(__ldg(reinterpret_cast<const __half*>(p))) * scale;
+        return __half2float(*reinterpret_cast<const __half*>(p)) * scale;
     else
-        return __ldg(p);
+        return *p;
 }
 
 template <class Cfg>
@@ -188,19 +229,19 @@ __device__ __forceinline__ unsigned float2_to_half2_bits(float a, float b)
     return u;
 }
 
-template <class Cfg>
+template <class Cfg, bool ORDERED = false>
 __device__ __forceinline__ V4<typename Cfg::real> ld_quad(const typename Cfg::pop* p)
 {
     if constexpr (Cfg::kHalf) {
-        const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+        const uint2 u = ld_state<ORDERED>(reinterpret_cast<const uint2*>(p));
         const float2 a = half2_bits_to_float2(u.x), b = half2_bits_to_float2(u.y);
         return {a.x, a.y, b.x, b.y};
     } else if constexpr (sizeof(typename Cfg::pop) == 8) {
-        const double2 a = __ldg(reinterpret_cast<const double2*>(p));
-        const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+        const double2 a = *reinterpret_cast<const double2*>(p);
+        const double2 b = reinterpret_cast<const double2*>(p)[1];
         return {a.x, a.y, b.x, b.y};
     } else {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 a = *reinterpret_cast<const float4*>(p);
         return {a.x, a.y, a.z, a.w};
     }
 }
@@ -220,17 +261,17 @@ __device__ __forceinline__ void st_quad(typename Cfg::pop* p, const V4<typename 
     }
 }
 
-template <class Cfg>
+template <class Cfg, bool ORDERED = false>
 __device__ __forceinline__ V2<typename Cfg::real> ld_fgpair(const typename Cfg::pop* p)
 {
     if constexpr (Cfg::kHalf) {
-        const float2 a = half2_bits_to_float2(__ldg(reinterpret_cast<const unsigned*>(p)));
+        const float2 a = half2_bits_to_float2(ld_state<ORDERED>(reinterpret_cast<const unsigned*>(p)));
         return {a.x, a.y};
     } else if constexpr (sizeof(typename Cfg::pop) == 8) {
-        const double2 a = __ldg(reinterpret_cast<const double2*>(p));
+        const double2 a = *reinterpret_cast<const double2*>(p);
         return {a.x, a.y};
     } else {
-        const float2 a = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 a = *reinterpret_cast<const float2*>(p);
         return {a.x, a.y};
     }
 }
@@ -275,7 +316,7 @@ __device__ __forceinline__ V2<typename Cfg::real> ld_pair_sh(const typename Cfg:
 
 // the three primitive 4-vectors of a cell (p at its first element of plane 0)
 // as 12 values in the order of the P_ indices; the planes are 4 stride apart
-template <class Cfg>
+template <class Cfg, bool ORDERED = false>
 __device__ __forceinline__ void ld_prims(const typename Cfg::prim* p, int64_t stride, typename Cfg::real (&v)[NPRIM])
 {
     using R = typename Cfg::real;
@@ -283,11 +324,11 @@ __device__ __forceinline__ void ld_prims(const typename Cfg::prim* p, int64_t st
     for (int q = 0; q < kPrimVecs; ++q) {
         const typename Cfg::prim* pq = p + 4 * q * stride;
         if constexpr (sizeof(typename Cfg::prim) == 8) {
-            const double2 a = __ldg(reinterpret_cast<const double2*>(pq));
-            const double2 b = __ldg(reinterpret_cast<const double2*>(pq) + 1);
+            const double2 a = *reinterpret_cast<const double2*>(pq);
+            const double2 b = reinterpret_cast<const double2*>(pq)[1];
             v[4 * q] = (R)a.x, v[4 * q + 1] = (R)a.y, v[4 * q + 2] = (R)b.x, v[4 * q + 3] = (R)b.y;
         } else {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(pq));
+            const float4 a = ld_state<ORDERED>(reinterpret_cast<const float4*>(pq));
             v[4 * q] = (R)a.x, v[4 * q + 1] = (R)a.y, v[4 * q + 2] = (R)a.z, v[4 * q + 3] = (R)a.w;
         }
     }
@@ -310,15 +351,15 @@ __device__ __forceinline__ void st_prims(typename Cfg::prim* p, int64_t stride, 
 }
 
 // a Maxwell pair (2m, 2m+1) at p
-template <class Cfg>
+template <class Cfg, bool ORDERED = false>
 __device__ __forceinline__ V2<typename Cfg::real> ld_hpair(const typename Cfg::hpop* p)
 {
     using R = typename Cfg::real;
     if constexpr (sizeof(typename Cfg::hpop) == 8) {
-        const double2 a = __ldg(reinterpret_cast<const double2*>(p));
+        const double2 a = *reinterpret_cast<const double2*>(p);
         return {(R)a.x, (R)a.y};
     } else {
-        const float2 a = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 a = ld_state<ORDERED>(reinterpret_cast<const float2*>(p));
         return {(R)a.x, (R)a.y};
     }
 }

@@ -122,10 +122,10 @@ __device__ __forceinline__ void train_outer(const float* d, const float* h, int 
 // each layer is one pass of 256 threads between two barriers. The one warp per
 // sample kernel before it read the weights from L1 at a stride (and added into
 // shared memory with 32-way bank conflicts): 164 us per batch of 1024, now 12 us.
-__global__ void __launch_bounds__(kTrainThreads) mlp_grad_kernel(const float* __restrict__ P,
+__global__ void __launch_bounds__(kTrainThreads) mlp_grad_kernel(const float* P,
                                                                  const float* __restrict__ data, int64_t n,
                                                                  int64_t count, uint64_t sample_seed,
-                                                                 float* __restrict__ partial, float inv_count)
+                                                                 float* partial, float inv_count)
 {
     extern __shared__ __align__(16) float sm[];
     const int t = threadIdx.x;
@@ -287,10 +287,9 @@ struct AdamStep {
 // own. 18 us a step of 1024 samples in all, 181 us before.
 constexpr int kReduceShares = 8;
 template <bool ADAM>
-__global__ void __launch_bounds__(32 * kReduceShares) mlp_reduce_kernel(const float* __restrict__ partial, int nblocks,
-                                                                        float* __restrict__ grad, float* __restrict__ P,
-                                                                        float* __restrict__ m, float* __restrict__ v,
-                                                                        float* __restrict__ loss, AdamStep a)
+__global__ void __launch_bounds__(32 * kReduceShares) mlp_reduce_kernel(const float* partial, int nblocks,
+                                                                                 float* grad, float* P, float* m, float* v,
+                                                                                 float* loss, AdamStep a)
 {
     __shared__ float sh[kReduceShares][32];
     const int lane = threadIdx.x % 32, share = threadIdx.x / 32, i = blockIdx.x * 32 + lane;

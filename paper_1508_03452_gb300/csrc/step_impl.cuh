@@ -413,13 +413,13 @@ struct StreamAll {
                                                R (&Tm)[10], R& Nm, R (&Na)[3])
     {
         if constexpr (G == 0) {
-            const V2<R> v = rest_pair<Cfg>(ld_fgpair<Cfg>(A.fgin + fg_elem(0, 0, c, A.stride)), A.hs);
+            const V2<R> v = rest_pair<Cfg>(ld_fgpair<Cfg, Cfg::kHalf>(A.fgin + fg_elem(0, 0, c, A.stride)), A.hs);
             store_group<0, Cfg, !IS3D>(V4<R>{v.x, v.y, R(0), R(0)}, S, Tm, Nm, Na);
         } else {
             const typename Cfg::pop* p = A.fgin + fg_elem(2 * G - 1, 0, c, A.stride);
             auto ld = [&](int a, int d) {
                 const int* oa = a == 0 ? o.x : (a == 1 ? o.y : o.z);
-                return ld_quad<Cfg>(d == 0 ? p : p + 4 * oa[d + 2]);
+                return ld_quad<Cfg, Cfg::kHalf>(d == 0 ? p : p + 4 * oa[d + 2]);
             };
             store_group<G, Cfg, !IS3D>(stream_group<G, IS3D, Cfg>(ld, A.k, A.hs), S, Tm, Nm, Na);
         }
@@ -476,7 +476,7 @@ struct PullH {
         constexpr int K = 2 * M;
         int off = o.x[2 - hop13(K, 0)] + o.y[2 - hop13(K, 1)];
         if (IS3D) off += o.z[2 - hop13(K, 2)];
-        const V2<R> hv = ld_hpair<Cfg>(A.hin + h_elem(K, c + off, A.stride));
+        const V2<R> hv = ld_hpair<Cfg, Cfg::kHalf>(A.hin + h_elem(K, c + off, A.stride));
         put_pair<R, Cfg::kVecSlots>(S.h(K), S.h(K + 1), hv.x, hv.y);
         acc_h_pair<M>(hv.x, hv.y, dEp, bn, rho);
         PullH<M + 1, IS3D, Cfg>::run(A, o, c, S, dEp, bn, rho);
@@ -1024,7 +1024,7 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
     } else {
         StreamAll<0, IS3D, Cfg>::run(A, o, c, S, Tm, Nm, Na);
         PullH<0, IS3D, Cfg>::run(A, o, c, S, dEp, bn, rho);
-        const R h24 = (R)A.hin[h_elem(24, c, A.stride)];
+        const R h24 = (R)ld_state<Cfg::kHalf>(A.hin + h_elem(24, c, A.stride));
         *S.h(24) = h24;
         rho += h24;
     }
@@ -1047,7 +1047,7 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
                 pv[4 * q] = (R)a.x, pv[4 * q + 1] = (R)a.y, pv[4 * q + 2] = (R)a.z, pv[4 * q + 3] = (R)a.w;
             }
         } else {
-            ld_prims<Cfg>(A.pin + prim_elem(0, c, A.stride), A.stride, pv);
+            ld_prims<Cfg, Cfg::kHalf>(A.pin + prim_elem(0, c, A.stride), A.stride, pv);
         }
         old.n = pv[P_N];
         old.eps = pv[P_EPS];
@@ -1419,10 +1419,8 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
 }
 
 // A programmatic launch (launch_step) may start while the kernel before it on the
-// stream drains; grid_wait returns when that has finished. grid_release comes after it:
-// when the next kernel's blocks launch, none runs that reads the buffer they read (the step
-// before last did; the boundary kernels release at their end), so no L1 line of it
-// outlives their launch.
+// stream drains; grid_wait returns when that has finished and its writes are visible to
+// this kernel's ordinary loads (ld_state), and grid_release comes after it.
 // one run: a 2-D grid of blocks over (x, y) and z
 template <class Cfg, bool IS3D, int SEED, bool OPEN>
 __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::value)
