@@ -48,7 +48,7 @@ NX = NY = 1024
 # primitives, each read once and written once
 BYTES_PER_CELL = {"fp64": 2 * (63 + 12) * 8, "fp32": 2 * (63 + 12) * 4, "fp16": 2 * (38 * 2 + 25 * 4 + 12 * 4)}
 PROFILE = os.path.join(ROOT, "profiles", "step_kernel_current_sheet_1024.md")
-KERNEL_SOURCES = ["step_impl.cuh", "lattice.cuh", "common.cuh", "mlp.cuh", "tma.cuh"]
+KERNEL_SOURCES = ["step_impl.cuh", "lattice.cuh", "common.cuh", "mlp.cuh", "mlp_tc.cuh", "tma.cuh"]
 GROUPS = {"n": (0,), "p": (1,), "eps": (2,), "u": (3, 4, 5), "E": (6, 7, 8), "B": (9, 10, 11)}
 
 
