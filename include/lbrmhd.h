@@ -304,7 +304,9 @@ int lbrmhd_lattice_tables(double* out, size_t n);
 /* ------------------------------------------------------------------------
  * Launch schedule of the runs of a handle. The paper runs one problem at a
  * time; the schedule only decides how the same cell updates are grouped into
- * kernel launches, so every schedule gives bit-identical results.
+ * kernel launches: in float64 every schedule gives bit-identical results, with every
+ * recovery seed; in float32 and float16 the schedules agree to the recovery tolerance
+ * (their kernels are compiled separately and may contract differently in the last bit).
  * ---------------------------------------------------------------------- */
 #define LBRMHD_SCHED_PER_RUN 0 /* one launch per run per step (a grid over the run's cells) */
 #define LBRMHD_SCHED_BATCH 1   /* one launch per step over the tiles of every run (per kernel variant:

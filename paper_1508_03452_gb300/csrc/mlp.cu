@@ -337,10 +337,7 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
         const int e = at + mlpd_frag_index(r, k, K);
         const __nv_bfloat16 b = __float2bfloat16_rn(v);
         W[STEP ? 4 * mlp_warp_order(e / 4) + e % 4 : e] = b;
-        if constexpr (STEP) {
-            if (!(tc == MLPT_W1 && k >= MLP_IN && k < MLP_IN + 3))  // (the bias inputs)
-                C[tc + mlpt_index(r, k, tc == MLPT_W2 || tc == MLPT_W3 ? MLPT_KB : K)] = b;
-        }
+        if constexpr (STEP) C[tc + mlpt_index(r, MLPT_KB + k, MLPT_KB + K)] = b;
     };
     const int total = MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H + MLPD_NBIAS;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
@@ -357,7 +354,7 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
         } else if (i < MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H) {
             const int j = i - MLP_H * MLP_K1 - 2 * MLP_H * MLP_H, r = j / MLP_H, k = j % MLP_H;
             put(MLPD_W4, MLPT_W4, r, k, MLP_H, r < MLP_OUT ? P[MLP_W4 + r * MLP_H + k] : 0.0f);
-            if constexpr (STEP) C[MLPT_W4 + mlpt_index(r + 8, k, MLP_H)] = __float2bfloat16_rn(0.0f);
+            if constexpr (STEP) C[MLPT_W4 + mlpt_index(r + 8, MLPT_KB + k, MLPT_K)] = __float2bfloat16_rn(0.0f);
         } else {
             const int j = i - (MLP_H * MLP_K1 + 2 * MLP_H * MLP_H + 8 * MLP_H);
             float val = 0.0f;
@@ -367,10 +364,8 @@ __global__ void mlp_pack_kernel(const float* __restrict__ P, unsigned char* __re
             else if (j < 192 + MLP_OUT) val = P[MLP_B4 + j - 192];
             bias[j] = val;
             if constexpr (STEP) {
-                if (j < 3 * MLP_H)
-                    mlpt_put_bias(C, j / MLP_H, j % MLP_H, val);
-                else if (j < 3 * MLP_H + MLP_OUT)
-                    reinterpret_cast<float*>(blob + MLPD_BYTES + MLPT_BIAS)[j - 3 * MLP_H] = val;
+                mlpt_put_bias(C, j / MLP_H, j % MLP_H, val);
+                if (j >= 3 * MLP_H) mlpt_put_bias(C, 3, j % MLP_H + 8, 0.0f);
             }
         }
     }

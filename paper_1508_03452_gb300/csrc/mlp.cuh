@@ -10,8 +10,7 @@
 // use warp-level bf16 tensor-core MMA (mma.sync m16n8k16, float32 accumulation): each
 // warp owns the 32 cells (rows) of its threads, so no block-wide barrier is needed and no
 // block holds tensor memory while it waits for another. The one-run step kernel uses
-// the tensor-memory form (mlp_tc.cuh); there a result a rounding away only starts the
-// eigen-solve elsewhere, where the standalone inference's is the user's.
+// the tensor-memory form (mlp_tc.cuh), whose sums agree with these bit for bit.
 #pragma once
 
 #include <cuda_bf16.h>

@@ -5,8 +5,8 @@
 // of the tile in both (lane t of the tensor memory). Its bf16 inputs are stored to
 // the operand columns, one thread issues the layer's products (operand A in tensor
 // memory, the weights in shared memory, float32 sums in tensor memory), and every
-// thread reads its row of sums back, adds the bias, applies the ReLU and stores the
-// next operand. What bounds it: the chain of four layers (store, products, commit,
+// thread reads its row of sums back, applies the ReLU and stores the next operand; the
+// biases start the sums, as products of constant inputs. What bounds it: the chain of four layers (store, products, commit,
 // load: ~700 clocks each), so several blocks share an SM; the products themselves
 // are a sixth of what mma.sync takes (one 128 x 64 x 16 product in ~34 clocks
 // against 128 mma.sync of 16).
@@ -23,15 +23,18 @@ constexpr int kTcOperand = 64;  // first operand column: 32 of activations, 8 of
 
 // Weights as the tensor core reads them from shared memory (K-major, no swizzle):
 // core matrices of 8 output rows x 8 inputs (8 rows of 16 bytes), those of a row
-// group side by side along K (128 bytes apart), row groups K * 16 bytes apart. Layer 1
-// takes the three bias inputs in its padding (inputs 20..22), layers 2 and 3 in 16
-// more inputs (64..66). The output layer is padded to 16 rows (the smallest N of a
-// 128-row product); its 4 float32 biases follow.
-constexpr int MLPT_KB = MLP_H + 16;  // inputs of layers 2 and 3
-constexpr int MLPT_W1 = 0, MLPT_W2 = MLPT_W1 + MLP_H * MLP_K1, MLPT_W3 = MLPT_W2 + MLP_H * MLPT_KB,
-              MLPT_W4 = MLPT_W3 + MLP_H * MLPT_KB, MLPT_NBF16 = MLPT_W4 + 16 * MLP_H;
-constexpr int MLPT_BIAS = MLPT_NBF16 * 2, MLPT_BYTES = MLPT_BIAS + MLP_OUT * 4;
-static_assert(MLPT_BYTES % 16 == 0 && MLPT_BIAS % 16 == 0, "one bulk copy, a vector load of the biases");
+// group side by side along K (128 bytes apart), row groups K * 16 bytes apart. The first
+// 16 inputs of a layer are the constants 1, 1, 1, 0, ..., whose weights add up to its
+// bias: their product starts the sums, as the bias starts those of the mma.sync form,
+// and the two forms' sums agree bit for bit (with the bias after the inputs, or added
+// to the outputs, a hidden unit's bf16 rounding could fall otherwise, and with it
+// the seed of a run depended on the launch schedule). The output layer is padded to 16
+// rows (the smallest N of a 128-row product).
+constexpr int MLPT_KB = 16;  // inputs of the bias
+constexpr int MLPT_K1 = MLPT_KB + MLP_K1, MLPT_K = MLPT_KB + MLP_H;
+constexpr int MLPT_W1 = 0, MLPT_W2 = MLPT_W1 + MLP_H * MLPT_K1, MLPT_W3 = MLPT_W2 + MLP_H * MLPT_K,
+              MLPT_W4 = MLPT_W3 + MLP_H * MLPT_K, MLPT_BYTES = 2 * (MLPT_W4 + 16 * MLPT_K);
+static_assert(MLPT_BYTES % 16 == 0, "one bulk copy");
 
 // element of weight (r, k) of a layer with K inputs, from the layer's start
 __host__ __device__ constexpr int mlpt_index(int r, int k, int K)
@@ -39,21 +42,20 @@ __host__ __device__ constexpr int mlpt_index(int r, int k, int K)
     return (r / 8) * (K * 8) + (k / 8) * 64 + (r % 8) * 8 + k % 8;
 }
 
-// the bias inputs' weights of hidden layer l (0..2), output r: three bf16 values
-// that add up to b exactly (an infinity or NaN as the first alone)
+// the bias inputs' weights of layer l (0..3), output r: three bf16 values, each
+// what the one before leaves of b, cut off, so that they add up to b exactly (an
+// infinity or NaN as the first alone)
 __device__ __forceinline__ void mlpt_put_bias(__nv_bfloat16* W, int l, int r, float b)
 {
-    const int K = l == 0 ? MLP_K1 : MLPT_KB, k = l == 0 ? MLP_IN : MLP_H;
-    __nv_bfloat16* w = W + (l == 0 ? MLPT_W1 : (l == 1 ? MLPT_W2 : MLPT_W3));
-    const __nv_bfloat16 b0 = __float2bfloat16_rn(b);
-    const float e = isfinite(__bfloat162float(b0)) ? b - __bfloat162float(b0) : 0.0f;
-    const __nv_bfloat16 b1 = __float2bfloat16_rn(e);
-    const float v[3] = {__bfloat162float(b0), __bfloat162float(b1), e - __bfloat162float(b1)};
+    const int K = l == 0 ? MLPT_K1 : MLPT_K;
+    __nv_bfloat16* w = W + (l == 0 ? MLPT_W1 : (l == 1 ? MLPT_W2 : (l == 2 ? MLPT_W3 : MLPT_W4)));
+    float rest = b;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) w[mlpt_index(r, k + j, K)] = __float2bfloat16_rn(v[j]);
-    if (l > 0)
-#pragma unroll
-        for (int j = 3; j < 16; ++j) w[mlpt_index(r, k + j, K)] = __float2bfloat16_rn(0.0f);
+    for (int j = 0; j < MLPT_KB; ++j) {
+        const float v = isfinite(rest) ? __uint_as_float(__float_as_uint(rest) & 0xffff0000u) : rest;
+        w[mlpt_index(r, j, K)] = __float2bfloat16_rn(j < 3 ? v : 0.0f);
+        rest = isfinite(rest) ? rest - v : 0.0f;
+    }
 }
 
 // --- tensor memory ----------------------------------------------------------
@@ -120,6 +122,7 @@ __device__ __forceinline__ void tc_ld4(uint32_t addr, float (&v)[4])
 
 // products of a layer: D (float32, 128 x N) = A (bf16, tensor memory, 128 x K) W^T,
 // then the commit that arrives on *bar (one thread)
+// (K with the bias inputs, which lie behind the activations in the operand)
 template <int K, int N>
 __device__ __forceinline__ void tc_layer(uint32_t tmem, uint32_t w_smem, uint64_t* bar)
 {
@@ -133,7 +136,7 @@ __device__ __forceinline__ void tc_layer(uint32_t tmem, uint32_t w_smem, uint64_
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
             "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem),
-            "r"(tmem + kTcOperand + 8 * k), "l"(desc), "r"(idesc), "r"(k)
+            "r"(tmem + kTcOperand + (k == 0 ? MLP_H / 2 : 8 * (k - 1))), "l"(desc), "r"(idesc), "r"(k)
             : "memory");
     }
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
@@ -157,7 +160,7 @@ __device__ __forceinline__ uint32_t pack_relu_bf16(float a, float b)  // (a in t
 
 constexpr uint32_t kTcOnes = 0x3f803f80u, kTcOne = 0x00003f80u;  // bf16 pairs (1, 1) and (1, 0)
 
-// the constant inputs of layers 2 and 3 (once per block, all of its threads)
+// the bias inputs (once per block, all of its threads)
 __device__ __forceinline__ void mlp_tc_constants(uint32_t tmem, int tid)
 {
     tc_st8(tmem + ((uint32_t)(tid & ~31) << 16) + kTcOperand + MLP_H / 2, kTcOnes, kTcOne, 0u);
@@ -186,7 +189,7 @@ __device__ __forceinline__ bool mlp_forward_tc(const uint32_t (&x)[MLP_IN / 2], 
     {
         uint32_t a[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) a[j] = j < MLP_IN / 2 ? x[j] : (j == MLP_IN / 2 ? kTcOnes : (j == MLP_IN / 2 + 1 ? kTcOne : 0u));
+        for (int j = 0; j < 16; ++j) a[j] = j < MLP_IN / 2 ? x[j] : 0u;
         tc_st16(mine + kTcOperand, a);
     }
 #pragma unroll
@@ -198,13 +201,13 @@ __device__ __forceinline__ bool mlp_forward_tc(const uint32_t (&x)[MLP_IN / 2], 
         if (tid == 0) {
             tc_fence_after();
             if (l == 0)
-                tc_layer<MLP_K1, MLP_H>(tmem, ws + 2 * MLPT_W1, bar);
+                tc_layer<MLPT_K1, MLP_H>(tmem, ws + 2 * MLPT_W1, bar);
             else if (l == 1)
-                tc_layer<MLPT_KB, MLP_H>(tmem, ws + 2 * MLPT_W2, bar);
+                tc_layer<MLPT_K, MLP_H>(tmem, ws + 2 * MLPT_W2, bar);
             else if (l == 2)
-                tc_layer<MLPT_KB, MLP_H>(tmem, ws + 2 * MLPT_W3, bar);
+                tc_layer<MLPT_K, MLP_H>(tmem, ws + 2 * MLPT_W3, bar);
             else
-                tc_layer<MLP_H, 16>(tmem, ws + 2 * MLPT_W4, bar);
+                tc_layer<MLPT_K, 16>(tmem, ws + 2 * MLPT_W4, bar);
         }
         ok = tc_wait(bar, phase);
         phase ^= 1u;
@@ -222,13 +225,53 @@ __device__ __forceinline__ bool mlp_forward_tc(const uint32_t (&x)[MLP_IN / 2], 
         }
     }
     tc_ld4(mine, y);
-    const float4 b = *reinterpret_cast<const float4*>(w + MLPT_BIAS);
-    y[0] += b.x;
-    y[1] += b.y;
-    y[2] += b.z;
-    y[3] += b.w;
     tc_fence_before();
     return __syncthreads_and(ok);  // every row has been read: the columns are free again
+}
+
+// A block's use of the network: tc_open takes its tensor memory and starts the copy of
+// the weights (all threads; a block barrier in it), tc_run takes the thread's row
+// through the network and gives the tensor memory back (all threads, once).
+struct TcCtx {
+    const unsigned char* w;  // weights in shared memory, arriving on bar[0]
+    uint64_t* bar;           // [0] the weights, [1] the products
+    uint32_t tmem;           // the block's columns
+};
+constexpr size_t kTcSmem = MLPT_BYTES + 3 * sizeof(uint64_t);  // weights, barriers, the columns' address
+
+__device__ __forceinline__ TcCtx tc_open(unsigned char* smem, const unsigned char* weights, int tid)
+{
+    TcCtx tm;
+    tm.w = smem;
+    tm.bar = reinterpret_cast<uint64_t*>(smem + MLPT_BYTES);
+    uint32_t* tmem_sh = reinterpret_cast<uint32_t*>(tm.bar + 2);
+    if (tid == 0) {
+        mbar_init(&tm.bar[0], 1u);
+        mbar_init(&tm.bar[1], 1u);
+        mbar_init_fence();
+        mbar_arrive_expect_tx(&tm.bar[0], MLPT_BYTES);
+        bulk_load(smem, weights, MLPT_BYTES, &tm.bar[0]);
+    }
+    if (tid < 32) tc_alloc(tmem_sh);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    tm.tmem = *tmem_sh;
+    mlp_tc_constants(tm.tmem, tid);
+    return tm;
+}
+
+__device__ __forceinline__ bool tc_run(const TcCtx& tm, const float (&feat)[MLP_IN], int tid, float (&y)[MLP_OUT])
+{
+    uint32_t xb[MLP_IN / 2];
+#pragma unroll
+    for (int j = 0; j < MLP_IN / 2; ++j) xb[j] = pack_bf16(feat[2 * j], feat[2 * j + 1]);
+    const bool in = mbar_wait_bounded(&tm.bar[0], 0u);
+    __syncwarp();
+    uint32_t phase = 0;
+    const bool got = mlp_forward_tc(xb, tm.w, tm.tmem, &tm.bar[1], phase, tid, y, in);
+    if (tid < 32) tc_dealloc(tm.tmem);
+    return got;
 }
 
 }  // namespace lb

@@ -960,13 +960,6 @@ struct TileStages<kTileStages, Cfg> {
     }
 };
 
-// The block's tensor-memory network (mlp_tc.cuh) in the one-run step kernel
-struct TcCtx {
-    const unsigned char* w;  // weights in shared memory, arriving on bar[0]
-    uint64_t* bar;           // [0] the weights, [1] the products
-    uint32_t tmem;           // the block's columns, given back after the network
-};
-
 // One cell update (x, y, z) of one run; `tid` is the thread's index in its
 // block of kStepThreads threads (its rows of the shared-memory buffers). Threads of
 // cells outside the grid return at once, except in the learned-seed variant,
@@ -1112,15 +1105,7 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
     if constexpr (SEED == SEED_MLP) {
         float out_f[MLP_OUT];
         if constexpr (TC) {
-            uint32_t xb[MLP_IN / 2];
-#pragma unroll
-            for (int j = 0; j < MLP_IN / 2; ++j) xb[j] = pack_bf16(feat[2 * j], feat[2 * j + 1]);
-            const bool in = mbar_wait_bounded(&tm->bar[0], 0u);
-            __syncwarp();
-            uint32_t phase = 0;
-            const bool got = mlp_forward_tc(xb, tm->w, tm->tmem, &tm->bar[1], phase, tid, out_f, in);
-            if (tid < 32) tc_dealloc(tm->tmem);
-            if (!got) {  // a wait ran out: the eigen-solve starts from the previous velocity
+            if (!tc_run(*tm, feat, tid, out_f)) {  // a wait ran out: the eigen-solve starts from the previous velocity
                 if (tid == 0) atomicOr(A.status, STATUS_TMA_TIMEOUT);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) out_f[a] = (float)(old.u[a] * k.inv_c);
@@ -1443,23 +1428,7 @@ __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::
         // flight while the block streams, the network's weights
         constexpr size_t slots = (size_t)kStepSlots * sizeof(typename Cfg::real) * kStepThreads;
         static_assert(slots % 16 == 0 && kStepThreads == kTcRows, "one row of the network per thread");
-        TcCtx tm;
-        tm.w = smem_raw + slots;
-        tm.bar = reinterpret_cast<uint64_t*>(smem_raw + slots + MLPT_BYTES);
-        uint32_t* tmem_sh = reinterpret_cast<uint32_t*>(tm.bar + 2);
-        if (tid == 0) {
-            mbar_init(&tm.bar[0], 1u);
-            mbar_init(&tm.bar[1], 1u);
-            mbar_init_fence();
-            mbar_arrive_expect_tx(&tm.bar[0], MLPT_BYTES);
-            bulk_load(smem_raw + slots, A.mlp + MLPD_BYTES, MLPT_BYTES, &tm.bar[0]);
-        }
-        if (tid < 32) tc_alloc(tmem_sh);
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        tm.tmem = *tmem_sh;
-        mlp_tc_constants(tm.tmem, tid);
+        const TcCtx tm = tc_open(smem_raw + slots, A.mlp + MLPD_BYTES, tid);
         step_cell<Cfg, IS3D, SEED, OPEN, false, kStepThreads, true>(A, x, y, z, tid, smem_raw, nullptr, &tm);
     } else {
         step_cell<Cfg, IS3D, SEED, OPEN>(A, x, y, z, tid, smem_raw);
@@ -1674,7 +1643,7 @@ __global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::
 template <class Cfg>
 size_t step_smem_bytes(int seed)
 {
-    return seed == SEED_MLP ? step_cell_smem<Cfg>(SEED_PREV) + MLPT_BYTES + 3 * sizeof(uint64_t) : step_cell_smem<Cfg>(seed);
+    return seed == SEED_MLP ? step_cell_smem<Cfg>(SEED_PREV) + kTcSmem : step_cell_smem<Cfg>(seed);
 }
 
 template <class Cfg>

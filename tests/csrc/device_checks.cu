@@ -1,0 +1,47 @@
+// Device functions of the library's headers behind plain C entries, for tests that
+// compare them on their own (tests/device_checks.py builds this file).
+#include "mlp_tc.cuh"
+
+namespace {
+
+// 128 rows a block through the tensor-memory network, as the one-run step kernel takes
+// its cells; rows past the end repeat the last one and are not stored
+__global__ void __launch_bounds__(lb::kTcRows) seed_kernel(const unsigned char* w, const float* feat, int64_t n, float* out,
+                                                           int* failed)
+{
+    __shared__ __align__(16) unsigned char sm[lb::kTcSmem];
+    const int tid = threadIdx.x;
+    const lb::TcCtx tm = lb::tc_open(sm, w, tid);
+    const int64_t row = blockIdx.x * (int64_t)lb::kTcRows + tid, r = row < n ? row : n - 1;
+    float x[lb::MLP_IN], y[lb::MLP_OUT];
+#pragma unroll
+    for (int j = 0; j < lb::MLP_IN; ++j) x[j] = feat[r * lb::MLP_IN + j];
+    if (!lb::tc_run(tm, x, tid, y)) {
+        if (tid == 0) atomicAdd(failed, 1);
+        return;
+    }
+    if (row < n)
+#pragma unroll
+        for (int j = 0; j < lb::MLP_OUT; ++j) out[row * lb::MLP_OUT + j] = y[j];
+}
+
+}  // namespace
+
+// blocks whose waits ran out (0 expected), or -1 on a CUDA error
+extern "C" int check_seed(const float* d_params, const float* d_feat, int64_t n, float* d_out)
+{
+    unsigned char* w = nullptr;
+    int* d_failed = nullptr;
+    int failed = -1;
+    if (n < 1 || cudaMalloc((void**)&w, lb::mlp_step_weight_bytes()) != cudaSuccess) return -1;
+    if (cudaMalloc((void**)&d_failed, sizeof(int)) == cudaSuccess && cudaMemset(d_failed, 0, sizeof(int)) == cudaSuccess &&
+        lb::launch_mlp_pack_step(d_params, w, nullptr) == cudaSuccess) {
+        seed_kernel<<<(unsigned)((n + lb::kTcRows - 1) / lb::kTcRows), lb::kTcRows>>>(w + lb::MLPD_BYTES, d_feat, n, d_out,
+                                                                                      d_failed);
+        if (cudaGetLastError() != cudaSuccess || cudaMemcpy(&failed, d_failed, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+            failed = -1;
+    }
+    cudaFree(d_failed);
+    cudaFree(w);
+    return failed;
+}
