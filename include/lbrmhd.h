@@ -54,8 +54,8 @@ extern "C" {
                                         cells keep their previous primitives, and lbrmhd_get_status returns
                                         this code */
 #define LBRMHD_ERR_NONFINITE (-5)    /* a NaN or Inf was found by the diagnostics */
-#define LBRMHD_ERR_TIMEOUT (-6)      /* a kernel's bounded wait for its own tile copies ran out (the block
-                                        skipped its update); returned by lbrmhd_get_status */
+#define LBRMHD_ERR_TIMEOUT (-6)      /* a kernel's bounded wait ran out; returned by lbrmhd_get_status, whose
+                                        status bits say which and what became of the update */
 #define LBRMHD_ERR_STATE (-7)        /* call out of order (e.g. step before init_fields) */
 
 /* boundary kinds, per face -x,+x,-y,+y,-z,+z */
@@ -266,8 +266,10 @@ int lbrmhd_get_stats(lbrmhd_handle h, int run, int64_t* out4);
  * NULL): [0] status bits raised by the step kernels since lbrmhd_create (1: a
  * TMA tile copy did not arrive within its wait limit, and that tile's update
  * was skipped; 2: a persistent launch's grid barrier gave up waiting, and the
- * launch's remaining steps were skipped), [1] recovery failures summed over every run since its
- * initialisation, [2] number of runs that step by the TMA tile kernel
+ * launch's remaining steps were skipped; 4: a block's network of the learned seed
+ * (PER_RUN schedule) did not finish within its wait limit, and the recoveries of its
+ * cells started from the previous velocity), [1] recovery failures summed over every
+ * run since its initialisation, [2] number of runs that step by the TMA tile kernel
  * (LBRMHD_FLAG_TMA_TILES).
  * Returns LBRMHD_ERR_TIMEOUT if a status bit is set, else
  * LBRMHD_ERR_NONCONVERGED if any recovery failed, else LBRMHD_OK; errors:

@@ -1470,6 +1470,8 @@ int lbrmhd_get_status(lbrmhd_handle h, int64_t* out3)
     }
     if (status & lb::STATUS_TMA_TIMEOUT) return fail(h, LBRMHD_ERR_TIMEOUT, "a TMA tile copy did not arrive in time");
     if (status & lb::STATUS_BARRIER_TIMEOUT) return fail(h, LBRMHD_ERR_TIMEOUT, "a grid barrier wait ran out");
+    if (status & lb::STATUS_SEED_TIMEOUT)
+        return fail(h, LBRMHD_ERR_TIMEOUT, "the learned seed's network did not finish in time (the recoveries started from the previous velocity)");
     if (fails > 0) return fail(h, LBRMHD_ERR_NONCONVERGED, std::to_string(fails) + " recoveries did not converge");
     return LBRMHD_OK;
 }

@@ -142,6 +142,7 @@ struct StepArgs {
 // status bits a step kernel can raise
 constexpr int STATUS_TMA_TIMEOUT = 1;      // a tile's copy did not arrive within the wait limit
 constexpr int STATUS_BARRIER_TIMEOUT = 2;  // a persistent launch's grid barrier gave up waiting
+constexpr int STATUS_SEED_TIMEOUT = 4;     // the learned seed's network did not finish within the wait limit
 // open_mask bit for runs that need the open-variant code without an open face
 constexpr int OPEN_EXTRA = 8;
 

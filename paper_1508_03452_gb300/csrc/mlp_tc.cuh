@@ -231,7 +231,8 @@ __device__ __forceinline__ bool mlp_forward_tc(const uint32_t (&x)[MLP_IN / 2], 
 
 // A block's use of the network: tc_open takes its tensor memory and starts the copy of
 // the weights (all threads; a block barrier in it), tc_run takes the thread's row
-// through the network and gives the tensor memory back (all threads, once).
+// through the network and gives the tensor memory back (all threads, once; false for
+// all of them if a wait ran out).
 struct TcCtx {
     const unsigned char* w;  // weights in shared memory, arriving on bar[0]
     uint64_t* bar;           // [0] the weights, [1] the products
@@ -270,6 +271,14 @@ __device__ __forceinline__ bool tc_run(const TcCtx& tm, const float (&feat)[MLP_
     __syncwarp();
     uint32_t phase = 0;
     const bool got = mlp_forward_tc(xb, tm.w, tm.tmem, &tm.bar[1], phase, tid, y, in);
+    if (!got) {
+        // a wait ran out: wait again, with a limit, for the copy and the products issued
+        // last, which must not outlive the block's memory (before the first products
+        // the parity is that of the barrier's past phase, and the wait returns at once)
+        mbar_wait_bounded(&tm.bar[0], 0u);
+        mbar_wait_bounded(&tm.bar[1], phase ^ 1u);
+        __syncwarp();
+    }
     if (tid < 32) tc_dealloc(tm.tmem);
     return got;
 }

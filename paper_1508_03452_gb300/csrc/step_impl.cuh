@@ -1106,7 +1106,7 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
         float out_f[MLP_OUT];
         if constexpr (TC) {
             if (!tc_run(*tm, feat, tid, out_f)) {  // a wait ran out: the eigen-solve starts from the previous velocity
-                if (tid == 0) atomicOr(A.status, STATUS_TMA_TIMEOUT);
+                if (tid == 0) atomicOr(A.status, STATUS_SEED_TIMEOUT);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) out_f[a] = (float)(old.u[a] * k.inv_c);
             }

@@ -25,7 +25,48 @@ __global__ void __launch_bounds__(lb::kTcRows) seed_kernel(const unsigned char* 
         for (int j = 0; j < lb::MLP_OUT; ++j) out[row * lb::MLP_OUT + j] = y[j];
 }
 
+// the same with weights that never arrive: the barrier expects their bytes, no copy is
+// started, and the block's waits run out; out counts the threads that were told so
+__global__ void __launch_bounds__(lb::kTcRows) late_seed_kernel(int* told)
+{
+    __shared__ __align__(16) unsigned char sm[lb::kTcSmem];
+    const int tid = threadIdx.x;
+    lb::TcCtx tm;
+    tm.w = sm;
+    tm.bar = reinterpret_cast<uint64_t*>(sm + lb::MLPT_BYTES);
+    uint32_t* columns = reinterpret_cast<uint32_t*>(tm.bar + 2);
+    if (tid == 0) {
+        lb::mbar_init(&tm.bar[0], 1u);
+        lb::mbar_init(&tm.bar[1], 1u);
+        lb::mbar_init_fence();
+        lb::mbar_arrive_expect_tx(&tm.bar[0], lb::MLPT_BYTES);
+    }
+    if (tid < 32) lb::tc_alloc(columns);
+    lb::tc_fence_before();
+    __syncthreads();
+    lb::tc_fence_after();
+    tm.tmem = *columns;
+    lb::mlp_tc_constants(tm.tmem, tid);
+    const float x[lb::MLP_IN] = {};
+    float y[lb::MLP_OUT];
+    if (!lb::tc_run(tm, x, tid, y)) atomicAdd(told, 1);
+}
+
 }  // namespace
+
+// threads of one block that were told that the weights did not arrive (128 expected)
+extern "C" int check_late_seed()
+{
+    int *d_told = nullptr, told = -1;
+    if (cudaMalloc((void**)&d_told, sizeof(int)) != cudaSuccess) return -1;
+    if (cudaMemset(d_told, 0, sizeof(int)) == cudaSuccess) {
+        late_seed_kernel<<<1, lb::kTcRows>>>(d_told);
+        if (cudaGetLastError() != cudaSuccess || cudaMemcpy(&told, d_told, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+            told = -1;
+    }
+    cudaFree(d_told);
+    return told;
+}
 
 // blocks whose waits ran out (0 expected), or -1 on a CUDA error
 extern "C" int check_seed(const float* d_params, const float* d_feat, int64_t n, float* d_out)
