@@ -74,15 +74,16 @@ struct HeqStore<24, Cfg, R> {
 };
 
 // Conversions between float32 and float64 on the integer pipes, the same values as
-// the conversion instructions: those share GB300's float64 pipe (two lanes per SM),
-// which bounds the passes below. Zeros and normal numbers are converted by shifts;
-// what is left (subnormals, infinities, NaN, overflow) takes the instruction.
+// the conversion instructions (which flush subnormal float32, -ftz=true): those share
+// GB300's float64 pipe (two lanes per SM), which bounds the passes below. All cases in
+// integers: an instruction in a rare branch is executed for every value, the compiler
+// turns the branch into a selection.
 __device__ __forceinline__ double widen(float v)
 {
     const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
-    if (m - 0x00800000u < 0x7f000000u)
-        return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
-    return m == 0u ? __hiloint2double((int)u, 0) : (double)v;
+    const unsigned hi = (m >> 3) + (m >= 0x7f800000u ? 0x70000000u : 0x38000000u);  // (infinity, NaN: all exponent bits)
+    const bool zero = m < 0x00800000u;
+    return __hiloint2double((int)((u & 0x80000000u) | (zero ? 0u : hi)), zero ? 0 : (int)(u << 29));
 }
 __device__ __forceinline__ double widen(double v) { return v; }
 
@@ -97,12 +98,14 @@ template <>
 __device__ __forceinline__ float narrow<float>(double v)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const unsigned hi = (unsigned)(b >> 32), e = (hi >> 20) & 0x7ffu;
-    if (e - 897u < 254u) {  // a normal float32: round to nearest even at bit 29, move the exponent
-        const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
-        return __uint_as_float((hi & 0x80000000u) | (((unsigned)(r >> 29) - 0xc0000000u) & 0x7fffffffu));
-    }
-    return (b << 1) == 0ull ? __uint_as_float(hi) : (float)v;
+    const unsigned hi = (unsigned)(b >> 32), m = hi & 0x7fffffffu;
+    // a normal float32: round to nearest even at bit 29 (up to infinity), move the exponent
+    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+    unsigned o = ((unsigned)(r >> 29) - 0xc0000000u) & 0x7fffffffu;
+    o = m < 0x38100000u ? 0u : o;           // below 2^-126
+    o = m >= 0x47f00000u ? 0x7f800000u : o;  // from 2^128 on, infinity
+    o = m > 0x7ff00000u || (m == 0x7ff00000u && (unsigned)b != 0u) ? 0x7fffffffu : o;  // NaN
+    return __uint_as_float((hi & 0x80000000u) | o);
 }
 
 template <class T>
@@ -111,8 +114,10 @@ __device__ __forceinline__ T narrow(FloatPair v)  // (float32 storage only)
     return (T)v.h;
 }
 // the type the initial state's equilibria are formed in: float64, or float32 pairs
-// where the results are stored as float32 (and float16): bit for bit what float64
-// gives, but for the rare value whose 48 bits do not settle the rounding to 24
+// where the results are stored as float32 (and float16). 48 bits are enough for sums
+// and products of deviations, not for what cancels to one: those are float64 in both
+// (set_equilibrium_init). The populations then are float64's deviations rounded to
+// float32, but for the rare value whose 48 bits do not settle the rounding.
 template <class Cfg>
 struct InitReal {
     using type = FloatPair;
@@ -190,37 +195,80 @@ __device__ __forceinline__ void heq_store_plane(const PopView<Cfg>& V, int64_t c
                       narrow<typename Cfg::real>(a[i] - x[i]));
 }
 
-// J from Eq. Ohm, g the Lorentz factor
+// J from Eq. Ohm, g the Lorentz factor; F = E + u x B and Eu = E.u / c^2, of which F
+// cancels in an ideal state and Eu across the flow
+__device__ __forceinline__ void ohm_terms(const double* E, const double* u, const double* B, double inv_c2, double* F,
+                                          double& Eu)
+{
+    Eu = (E[0] * u[0] + E[1] * u[1] + E[2] * u[2]) * inv_c2;
+    F[0] = fma(u[1], B[2], fma(-u[2], B[1], E[0]));
+    F[1] = fma(u[2], B[0], fma(-u[0], B[2], E[1]));
+    F[2] = fma(u[0], B[1], fma(-u[1], B[0], E[2]));
+}
 template <class Q>
-__device__ __forceinline__ void ohm_current_g(const Q* E, const Q* u, const Q* B, Q rho, Q g, const Phys<Q>& k, Q* J)
+__device__ __forceinline__ void ohm_current_terms(const Q* F, Q Eu, const Q* u, Q rho, Q g, const Phys<Q>& k, Q* J)
 {
     const Q sg = k.sigma * g;
-    const Q Eu = (E[0] * u[0] + E[1] * u[1] + E[2] * u[2]) * (k.inv_c * k.inv_c);
-    const Q F[3] = {fma(u[1], B[2], fma(-u[2], B[1], E[0])), fma(u[2], B[0], fma(-u[0], B[2], E[1])),
-                    fma(u[0], B[1], fma(-u[1], B[0], E[2]))};
     for (int a = 0; a < 3; ++a) J[a] = fma(rho, u[a], sg * fma(-Eu, u[a], F[a]));
 }
-
-// every population of cell c at its equilibrium for primitives s
-template <class Cfg, class Q>
-__device__ __forceinline__ void set_equilibrium_init(const PopView<Cfg>& V, int64_t c, const Prim<Q>& s, const Phys<Q>& k)
+__device__ __forceinline__ void ohm_current_g(const double* E, const double* u, const double* B, double rho, double g,
+                                              const Phys<double>& k, double* J)
 {
-    const Q b2 = (s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2]) * (k.inv_c * k.inv_c);
+    double F[3], Eu;
+    ohm_terms(E, u, B, k.inv_c * k.inv_c, F, Eu);
+    ohm_current_terms(F, Eu, u, rho, g, k, J);
+}
+
+// the constants of a run that the initial state's float64 differences take
+struct InitPhys {
+    double c2, inv_c2, gm1, inv_gm1, eps0_2dx, n_r, eps_r, Er[3], Br[3];
+};
+inline InitPhys init_consts(const Phys<double>& k)
+{
+    return {k.c2,    k.inv_c * k.inv_c, k.gm1, 1.0 / k.gm1, k.eps0 / (2.0 * k.dx), k.n_r, k.eps_r, {k.Er[0], k.Er[1], k.Er[2]},
+            {k.Br[0], k.Br[1], k.Br[2]}};
+}
+
+// Every population of cell c at its equilibrium for primitives s. The deviations from
+// the reference state, the pressure's, 1 - u^2 / c^2 and Ohm's E + u x B are
+// differences of near-equal numbers: float64, and only then of type Q. (With the
+// differences taken in float32 pairs a deviation of relative size d was wrong by
+// ~2e-15 / d of itself, and J of an ideal state by ~2e-15 sigma |u| |B|.)
+template <class Cfg, class Q>
+__device__ __forceinline__ void set_equilibrium_init(const PopView<Cfg>& V, int64_t c, const Prim<double>& s,
+                                                     const InitPhys& w, const Phys<Q>& k)
+{
+    const double n_dev = s.n - w.n_r, eps_dev = s.eps - w.eps_r;
+    const Q p_dev = split<Q>(w.gm1 * (eps_dev - n_dev * w.c2));
+    const double b2 = (s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2]) * w.inv_c2;
     Lorentz<Q> lz;
-    lz.g = rsqrt_newton(Q(1) - b2);
+    lz.g = rsqrt_newton(split<Q>(1.0 - b2));
     lz.g2 = lz.g * lz.g;
-    lz.gm1 = lz.g2 * b2 * rcp_approx(lz.g + Q(1));
-    Q J[3];
-    ohm_current_g(s.E, s.u, s.B, s.rho, lz.g, k, J);
-    const Q dE[3] = {s.E[0] - k.Er[0], s.E[1] - k.Er[1], s.E[2] - k.Er[2]};
-    const Q dB[3] = {s.B[0] - k.Br[0], s.B[1] - k.Br[1], s.B[2] - k.Br[2]};
+    lz.gm1 = lz.g2 * split<Q>(b2) * rcp_approx(lz.g + Q(1));
+    double F[3], Eu;
+    ohm_terms(s.E, s.u, s.B, w.inv_c2, F, Eu);
+    Prim<Q> q;
+    q.n = split<Q>(s.n);
+    q.eps = split<Q>(s.eps);
+    q.rho = split<Q>(s.rho);
+    Q J[3], Fq[3], dE[3], dB[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        q.u[a] = split<Q>(s.u[a]);
+        q.E[a] = split<Q>(s.E[a]);
+        q.B[a] = split<Q>(s.B[a]);
+        Fq[a] = split<Q>(F[a]);
+        dE[a] = split<Q>(s.E[a] - w.Er[a]);
+        dB[a] = split<Q>(s.B[a] - w.Br[a]);
+    }
+    ohm_current_terms(Fq, split<Q>(Eu), q.u, q.rho, lz.g, k, J);
     heq_store_plane<0, Cfg>(V, c, dE, dB, J, k);
     heq_store_plane<1, Cfg>(V, c, dE, dB, J, k);
     heq_store_plane<2, Cfg>(V, c, dE, dB, J, k);
-    EqCell<Q> q;
-    eq_cell(s, s.n - k.n_r, s.eps - k.eps_r, dE, dB, k, q, &lz);
+    EqCell<Q> eq;
+    eq_cell(q, split<Q>(n_dev), split<Q>(eps_dev), dE, dB, k, eq, &lz, &p_dev);
     EqEvenT<Q> e;
-    eq_even(q, e);
+    eq_even(eq, e);
     EqStoreEven<0, Cfg, Q>::run(V, c, e);
 }
 
@@ -270,13 +318,13 @@ __device__ __forceinline__ double input_E1(const InitInputs& in, int64_t c, int6
 // Bound by arithmetic, in float64 by GB300's rate of two lanes per SM: opposite
 // directions share the even and odd parts of their equilibria, a plane's Maxwell pairs
 // their sums, one Lorentz factor serves J and the equilibria, and where the results
-// are stored in float32 all but E and div E is in float32 pairs. 256^3
+// are stored in float32 all but E, div E and what cancels is in float32 pairs. 256^3
 // cells in float32: 21.5 ms direction by direction in float64, 14.3 with the terms
-// shared, 5.7 with the pairs (memory would take 0.9).
+// shared, 4.9 with the pairs (memory would take 0.9; 9.3 with the conversions' rare cases
+// left to the instructions).
 template <class Cfg>
 __global__ void __launch_bounds__(128) init_kernel(PopView<Cfg> V, InitInputs in, Phys<typename InitReal<Cfg>::type> k,
-                                                   double c2, double inv_gm1, double eps0_2dx, int* bad)
-
+                                                   InitPhys w, int* bad)
 {
     const int64_t N = (int64_t)V.nx * V.ny * V.nz;
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -284,13 +332,17 @@ __global__ void __launch_bounds__(128) init_kernel(PopView<Cfg> V, InitInputs in
     const int x = (int)(c % V.nx), y = (int)((c / V.nx) % V.ny), z = (int)(c / ((int64_t)V.nx * V.ny));
     Prim<double> s;
     s.n = in.n[c];
-    s.eps = s.n * c2 + in.p[c] * inv_gm1;
+    // p / (Gamma - 1): the product with the reciprocal, corrected by its remainder (as the
+    // division rounds; an infinite p has no remainder)
+    const double p = in.p[c], pq = p * w.inv_gm1;
+    const bool over = ((unsigned)__double2hiint(pq) & 0x7ff00000u) == 0x7ff00000u;
+    s.eps = s.n * w.c2 + (over ? pq : fma(fma(-pq, w.gm1, p), w.inv_gm1, pq));
     for (int a = 0; a < 3; ++a) {
         s.u[a] = in.u[a * N + c];
         s.B[a] = in.B[a * N + c];
     }
     input_E(in, c, N, s.E);
-    if (!(s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2] < c2) || !(s.n > 0)) atomicExch(bad, 1);
+    if (!(s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2] < w.c2) || !(s.n > 0)) atomicExch(bad, 1);
     // rho_c = eps0 div E
     double div = 0.0;
     if (V.nx > 1) {
@@ -308,7 +360,7 @@ __global__ void __launch_bounds__(128) init_kernel(PopView<Cfg> V, InitInputs in
         div += input_E1<2>(in, col + plane * wrap_coord(z + 1, V.nz, V.periodic[2]), N) -
                input_E1<2>(in, col + plane * wrap_coord(z - 1, V.nz, V.periodic[2]), N);
     }
-    s.rho = eps0_2dx * div;
+    s.rho = w.eps0_2dx * div;
     {
         typename Cfg::prim pv[NPRIM];
         pv[P_N] = narrow<typename Cfg::prim>(s.n);
@@ -323,18 +375,7 @@ __global__ void __launch_bounds__(128) init_kernel(PopView<Cfg> V, InitInputs in
         st_prims<Cfg>(V.prim + prim_elem(0, c, V.stride), V.stride, pv);
     }
     V.h[h_elem(24, c, V.stride)] = narrow<typename Cfg::hpop>(s.rho);
-    using Q = typename InitReal<Cfg>::type;
-    Prim<Q> sq;
-    sq.n = split<Q>(s.n);
-    sq.eps = split<Q>(s.eps);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        sq.u[a] = split<Q>(s.u[a]);
-        sq.E[a] = split<Q>(s.E[a]);
-        sq.B[a] = split<Q>(s.B[a]);
-    }
-    sq.rho = split<Q>(s.rho);
-    set_equilibrium_init<Cfg, Q>(V, c, sq, k);
+    set_equilibrium_init<Cfg>(V, c, s, w, k);
 }
 
 // float64 means for the reference state: n, p, E (3), B (3), E_a E_b (6: xx yy
@@ -569,8 +610,8 @@ __global__ void prim_component_kernel(PopView<Cfg> V, int P, typename Cfg::prim*
 
 
 // Bound by the float64 rate, not by memory (176 bytes a cell in float32): ~35 float64
-// instructions a cell, the conversions on the integer pipes. 1024^2 121 -> 82 us, 2048^2
-// float16 475 -> 274 us.
+// instructions a cell, the conversions on the integer pipes. 1024^2 121 -> 65 us, 2048^2
+// float16 475 -> 250 us.
 template <class Cfg>
 __global__ void __launch_bounds__(128) moments_kernel(PopView<Cfg> V, Phys<double> k, double* out)
 {
@@ -830,8 +871,8 @@ cudaError_t launch_init(const PopView<Cfg>& V, const InitInputs& in, const Phys<
                         cudaStream_t s)
 {
     const int64_t N = (int64_t)V.nx * V.ny * V.nz;
-    init_kernel<Cfg><<<blocks_for(N, 128), 128, 0, s>>>(V, in, init_phys(k, typename InitReal<Cfg>::type{}), k.c2, 1.0 / k.gm1,
-                                                        k.eps0 / (2.0 * k.dx), bad);
+    init_kernel<Cfg><<<blocks_for(N, 128), 128, 0, s>>>(V, in, init_phys(k, typename InitReal<Cfg>::type{}), init_consts(k),
+                                                        bad);
     return cudaGetLastError();
 }
 

@@ -176,19 +176,21 @@ struct EqCell {
     R kf, kq[3];
 };
 
-// (lz: the Lorentz factor where the caller has it, else it is formed here)
+// (lz, p_given: the Lorentz factor and p - p_r where the caller has them, else they are
+// formed here)
 // n_dev = n - n_r, eps_dev = eps - eps_r, dE = E - Er and dB = B - Br are passed
 // separately so that the float32 path never rounds the large reference values
 // into the deviations.
 template <class R>
 __device__ __forceinline__ void eq_cell(const Prim<R>& s, R n_dev, R eps_dev, const R* dE, const R* dB,
-                                        const Phys<R>& k, EqCell<R>& q, const Lorentz<R>* lz = nullptr)
+                                        const Phys<R>& k, EqCell<R>& q, const Lorentz<R>* lz = nullptr,
+                                        const R* p_given = nullptr)
 {
     const R b[3] = {s.u[0] * k.inv_c, s.u[1] * k.inv_c, s.u[2] * k.inv_c};
     const R b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
     const R g2 = lz ? lz->g2 : R(1) / (R(1) - b2);
     const R g = lz ? lz->g : sqrt(g2);
-    const R p_dev = k.gm1 * (eps_dev - n_dev * k.c2);
+    const R p_dev = p_given ? *p_given : k.gm1 * (eps_dev - n_dev * k.c2);
     const R three_dp = R(3) * p_dev;
     const R rest_dev = R(kRest) * (R(3) * p_dev - eps_dev);
     const R wq = R(0.75) * (s.eps + k.p_r + p_dev);
