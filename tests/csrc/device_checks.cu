@@ -1,5 +1,6 @@
 // Device functions of the library's headers behind plain C entries, for tests that
 // compare them on their own (tests/device_checks.py builds this file).
+#include "lattice.cuh"
 #include "mlp_tc.cuh"
 
 namespace {
@@ -52,7 +53,23 @@ __global__ void __launch_bounds__(lb::kTcRows) late_seed_kernel(int* told)
     if (!lb::tc_run(tm, x, tid, y)) atomicAdd(told, 1);
 }
 
+__global__ void reciprocal_kernel(const double* x, int64_t n, double* rcp, double* rsqrt)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    rcp[i] = lb::rcp_approx(x[i]);
+    rsqrt[i] = lb::rsqrt_newton(x[i]);
+}
+
 }  // namespace
+
+// the float64 reciprocals of n values; 0, or -1 on a CUDA error
+extern "C" int check_reciprocals(const double* d_x, int64_t n, double* d_rcp, double* d_rsqrt)
+{
+    if (n < 1) return -1;
+    reciprocal_kernel<<<(unsigned)((n + 127) / 128), 128>>>(d_x, n, d_rcp, d_rsqrt);
+    return cudaGetLastError() == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess ? 0 : -1;
+}
 
 // threads of one block that were told that the weights did not arrive (128 expected)
 extern "C" int check_late_seed()
