@@ -473,12 +473,15 @@ bool train_configured()
     return ok;
 }
 
-// blocks of a gradient: one per kTS samples, up to three per SM of the 152 (the
-// shared memory holds three), each then walking several tiles
+// blocks of a gradient: one per kTS samples, up to a fixed number (three for each SM of a
+// GB300, which is what the shared memory holds), each then walking several tiles. Fixed,
+// not asked of the device: it sets the order in which a gradient is summed, and a
+// training run's bits are not to depend on where it runs.
+constexpr int kTrainBlocks = 456;
 int g_train_blocks(int64_t count)
 {
     const int64_t b = (count + lb::kTS - 1) / lb::kTS;
-    return (int)(b < 1 ? 1 : (b > 456 ? 456 : b));
+    return (int)(b < 1 ? 1 : (b > kTrainBlocks ? kTrainBlocks : b));
 }
 
 // launches a kernel that, unless it is the `first` of a call, may start while its
@@ -580,7 +583,7 @@ int lbrmhd_mlp_infer(const void* d_blob, const float* d_features, int64_t n, flo
 {
     if (!d_blob || !d_features || !d_out || n < 0) return LBRMHD_ERR_BAD_ARG;
     if (n == 0) return LBRMHD_OK;
-    const int64_t grid = 152 * lb::kInferBlocks;  // one wave
+    const int64_t grid = (int64_t)lb::device_sms() * lb::kInferBlocks;  // one wave
     const int64_t tiles = (n + 31) / 32, blocks = (tiles + lb::kInferWarps - 1) / lb::kInferWarps;
     lb::mlp_infer_kernel<<<(unsigned)(blocks < grid ? blocks : grid), 32 * lb::kInferWarps, 0, (cudaStream_t)stream>>>(
         (const unsigned char*)d_blob, d_features, n, d_out);

@@ -1897,7 +1897,7 @@ cudaError_t launch_step(const StepArgs<Cfg>& A, cudaStream_t stream, const TileL
     // SM's float64 lanes (377 steps of a 100-cell line 31.8 -> 30.6 ms; float32 runs of
     // 128 warps gained nothing, and such blocks or narrower rows cost a sweep of runs
     // 96 to 384 wide 20 %)
-    if (sizeof(typename Cfg::real) == 8 && A.seed != SEED_MLP && (int64_t)((A.nx + 31) / 32) * A.ny * A.nz <= 152) {
+    if (sizeof(typename Cfg::real) == 8 && A.seed != SEED_MLP && (int64_t)((A.nx + 31) / 32) * A.ny * A.nz <= device_sms()) {
         bx = 32;
         by = 1;
     }

@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace lb {
 
 constexpr unsigned long long kTmaWaitNs = 500ull * 1000ull * 1000ull;  // 0.5 s
@@ -85,6 +87,19 @@ __device__ __forceinline__ unsigned long long global_ns()
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+
+// multiprocessors of the current device (read once per device)
+inline int device_sms()
+{
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (dev < kDevices && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+    if (dev < kDevices) known[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 // the grid's predecessor on the stream has finished and its writes are visible
