@@ -693,8 +693,10 @@ constexpr int kStepSlots = 63;  // 19 f + 19 g + 25 h pre-collision values per c
 #define LB_STEP_BX 128  // block width along x (the block is LB_STEP_BX x 128 / LB_STEP_BX)
 #endif
 #ifndef LB_STEP_MIN_BLOCKS_F16
-// float16-deviation storage, 2-D: 5 blocks (102 registers) against 4 of 128, 10 steps and
-// a read-out of 2048^2 4.90 -> 4.81 ms (with more instructions in the stencil 4 won)
+// float16-deviation storage, 2-D: 5 blocks (96 registers) against 4 of 128, where a grid
+// is more than 4 blocks an SM: 10 steps and a read-out of 2048^2 4.83 against 4.89 ms;
+// 1024^2 in a batched launch 220 against 260 us a step, in a persistent one 211 against
+// 247 (StepRoomyBlocks for smaller grids)
 #define LB_STEP_MIN_BLOCKS_F16 5
 #endif
 #ifndef LB_STEP_MIN_BLOCKS_F16_3D
@@ -712,6 +714,16 @@ struct StepMinBlocks {
                                  : Cfg::kHalf                   ? LB_STEP_MIN_BLOCKS_F16
                                  : IS3D                         ? LB_STEP_MIN_BLOCKS_3D
                                                                 : LB_STEP_MIN_BLOCKS;
+};
+
+// Resident blocks for a grid that fits an SM's registers at fewer of them: a fifth block has
+// nothing to run then and costs registers (six float16 runs of 100 x 60 cells, us a step:
+// batched 14.5 against 16.5, persistent 13.5 against 14.4, run by run 38.5 against 40).
+template <class Cfg, int SEED, bool IS3D>
+struct StepRoomyBlocks {
+    static constexpr int value = Cfg::kHalf && !IS3D && SEED != SEED_MLP ? 4 : StepMinBlocks<Cfg, SEED, IS3D>::value;
+    static constexpr bool differs = value != StepMinBlocks<Cfg, SEED, IS3D>::value;
+    static bool fits(int64_t grid) { return differs && grid <= (int64_t)value * device_sms(); }
 };
 
 // Photospheric body force (reading R25) on the streamed f of one cell: the
@@ -1407,8 +1419,8 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
 // stream drains; grid_wait returns when that has finished and its writes are visible to
 // this kernel's ordinary loads (ld_state), and grid_release comes after it.
 // one run: a 2-D grid of blocks over (x, y) and z
-template <class Cfg, bool IS3D, int SEED, bool OPEN>
-__global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::value)
+template <class Cfg, bool IS3D, int SEED, bool OPEN, int BLOCKS = StepMinBlocks<Cfg, SEED, IS3D>::value>
+__global__ void __launch_bounds__(kStepThreads, BLOCKS)
     step_kernel(const StepArgs<Cfg> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1546,8 +1558,8 @@ __host__ __device__ constexpr size_t batch_args_bytes()
 // (persistent when the grid is one wave of resident blocks). A block copies
 // the arguments of a tile's run from device memory into shared memory when
 // the run changes from its previous tile.
-template <class Cfg, bool IS3D, int SEED, bool OPEN>
-__global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::value)
+template <class Cfg, bool IS3D, int SEED, bool OPEN, int BLOCKS = StepMinBlocks<Cfg, SEED, IS3D>::value>
+__global__ void __launch_bounds__(kStepThreads, BLOCKS)
     step_batch_kernel(const unsigned char* __restrict__ args, const int4* __restrict__ tiles, int ntiles, int bx)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1608,8 +1620,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int
     return __syncthreads_and(ok) != 0;
 }
 
-template <class Cfg, bool IS3D, int SEED, bool OPEN>
-__global__ void __launch_bounds__(kStepThreads, StepMinBlocks<Cfg, SEED, IS3D>::value)
+template <class Cfg, bool IS3D, int SEED, bool OPEN, int BLOCKS = StepMinBlocks<Cfg, SEED, IS3D>::value>
+__global__ void __launch_bounds__(kStepThreads, BLOCKS)
     step_persistent_kernel(const unsigned char* __restrict__ args, size_t parity_bytes, int in0,
                            const int4* __restrict__ tiles, int ntiles, int bx, int nsteps, unsigned int* counter,
                            int* status, unsigned long long wait_ns)
@@ -1685,6 +1697,15 @@ struct SetSmemAttr {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(step_batch_kernel<Cfg, D, S, O>, a, (int)batch_smem_bytes<Cfg>(S));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(step_persistent_kernel<Cfg, D, S, O>, a, (int)batch_smem_bytes<Cfg>(S));
+        using Roomy = StepRoomyBlocks<Cfg, S, D>;
+        if constexpr (Roomy::differs) {
+            constexpr int B = Roomy::value;
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel<Cfg, D, S, O, B>, a, (int)step_smem_bytes<Cfg>(S));
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(step_batch_kernel<Cfg, D, S, O, B>, a, (int)batch_smem_bytes<Cfg>(S));
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(step_persistent_kernel<Cfg, D, S, O, B>, a, (int)batch_smem_bytes<Cfg>(S));
+        }
         return e;
     }
 };
@@ -1750,7 +1771,9 @@ struct LaunchBatch {
     template <bool D, int S, bool O>
     cudaError_t run()
     {
-        step_batch_kernel<Cfg, D, S, O><<<grid, kStepThreads, batch_smem_bytes<Cfg>(S), stream>>>(args, tiles, ntiles, bx);
+        using Roomy = StepRoomyBlocks<Cfg, S, D>;
+        auto kernel = Roomy::fits(grid) ? step_batch_kernel<Cfg, D, S, O, Roomy::value> : step_batch_kernel<Cfg, D, S, O>;
+        kernel<<<grid, kStepThreads, batch_smem_bytes<Cfg>(S), stream>>>(args, tiles, ntiles, bx);
         return cudaGetLastError();
     }
 };
@@ -1802,8 +1825,11 @@ struct LaunchPersistent {
         at[0].val.cooperative = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, step_persistent_kernel<Cfg, D, S, O>, args, parity_bytes, in0, tiles, ntiles,
-                                  bx, nsteps, counter, status, wait_ns);
+        using Roomy = StepRoomyBlocks<Cfg, S, D>;  // (every block stays resident: the grid fits at its blocks an SM)
+        auto kernel =
+            Roomy::fits(grid) ? step_persistent_kernel<Cfg, D, S, O, Roomy::value> : step_persistent_kernel<Cfg, D, S, O>;
+        return cudaLaunchKernelEx(&cfg, kernel, args, parity_bytes, in0, tiles, ntiles, bx, nsteps, counter, status,
+                                  wait_ns);
     }
 };
 
@@ -1856,7 +1882,9 @@ struct LaunchRun {
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
         cfg.numAttrs = overlap ? 1 : 0;
-        return cudaLaunchKernelEx(&cfg, step_kernel<Cfg, D, S, O>, *A);
+        using Roomy = StepRoomyBlocks<Cfg, S, D>;
+        const bool roomy = Roomy::fits((int64_t)grid.x * grid.y * grid.z);
+        return cudaLaunchKernelEx(&cfg, roomy ? step_kernel<Cfg, D, S, O, Roomy::value> : step_kernel<Cfg, D, S, O>, *A);
     }
 };
 
