@@ -670,13 +670,6 @@ __device__ __forceinline__ void collide_h_plane(const StepArgs<Cfg>& A, int64_t 
     }
 }
 
-// 16-row tiles of a warp's 32 cells that the learned seed takes through the network
-// at a time: 1 (231 us a step of the 1024^2 sheet), because two tiles' fragments
-// beside the cell's state spill (239 us) though they read the weights once
-#ifndef LB_MLP_TILES
-#define LB_MLP_TILES 1
-#endif
-constexpr int kMlpTiles = LB_MLP_TILES;
 constexpr int kStepSlots = 63;  // 19 f + 19 g + 25 h pre-collision values per cell in shared memory
 #ifndef LB_STEP_MIN_BLOCKS
 // resident 128-thread blocks per SM targeted for 2-D runs in float32 storage:
@@ -703,7 +696,10 @@ constexpr int kStepSlots = 63;  // 19 f + 19 g + 25 h pre-collision values per c
 #define LB_STEP_MIN_BLOCKS_F16_3D 4
 #endif
 #ifndef LB_STEP_MIN_BLOCKS_MLP
-#define LB_STEP_MIN_BLOCKS_MLP 3  // the learned-seed variant: 3 blocks (168 registers) beat 4 by 1 %, 2 by 23 %
+// the learned-seed variant: 3 blocks (168 registers); 10 steps of the 1024^2 sheet by the one-run
+// kernel 2.10 ms, with 4 blocks 2.22, with 2 2.68 (the batched kernels gain from a fourth, seven
+// runs 691 -> 578 us a step, and six small ones lose a tenth)
+#define LB_STEP_MIN_BLOCKS_MLP 3
 #endif
 // float64: 2 blocks
 template <class Cfg, int SEED, bool IS3D = false>
@@ -1132,19 +1128,20 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
                     __floats2bfloat162_rn(j < MLP_IN ? feat[j] : 0.0f, j + 1 < MLP_IN ? feat[j + 1] : 0.0f);
             __syncwarp();
             const int lane = tid & 31;
+            // 16 rows of the warp's 32 cells at a time: both at once read the weights once, but
+            // their fragments beside the cell's state spill (seven runs, batched 692 us a step
+            // against 708, persistent 667 against 688)
 #pragma unroll
-            for (int part = 0; part < 2 / kMlpTiles; ++part) {
-                __nv_bfloat16* rows = act + ((tid & ~31) + 16 * kMlpTiles * part) * MLP_FROW;
-                float y[kMlpTiles][4];
-                mlp_forward_frag<kMlpTiles, true>(rows, A.mlp, y);
+            for (int part = 0; part < 2; ++part) {
+                __nv_bfloat16* rows = act + ((tid & ~31) + 16 * part) * MLP_FROW;
+                float y[1][4];
+                mlp_forward_frag<1, true>(rows, A.mlp, y);
                 __syncwarp();  // the feature rows have been read: the outputs take their place
                 if ((lane & 3) < 2)
 #pragma unroll
-                    for (int mt = 0; mt < kMlpTiles; ++mt)
-#pragma unroll
-                        for (int hh = 0; hh < 2; ++hh)
-                            *reinterpret_cast<float2*>(rows + (16 * mt + (lane >> 2) + 8 * hh) * MLP_FROW + 4 * (lane & 3)) =
-                                make_float2(y[mt][2 * hh], y[mt][2 * hh + 1]);
+                    for (int hh = 0; hh < 2; ++hh)
+                        *reinterpret_cast<float2*>(rows + ((lane >> 2) + 8 * hh) * MLP_FROW + 4 * (lane & 3)) =
+                            make_float2(y[0][2 * hh], y[0][2 * hh + 1]);
             }
             __syncwarp();
             const float* out = reinterpret_cast<const float*>(row);
