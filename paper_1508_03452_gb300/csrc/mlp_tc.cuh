@@ -6,10 +6,10 @@
 // the operand columns, one thread issues the layer's products (operand A in tensor
 // memory, the weights in shared memory, float32 sums in tensor memory), and every
 // thread reads its row of sums back, applies the ReLU and stores the next operand; the
-// biases start the sums, as products of constant inputs. What bounds it: the chain of four layers (store, products, commit,
-// load: ~700 clocks each), so several blocks share an SM; the products themselves
-// are a sixth of what mma.sync takes (one 128 x 64 x 16 product in ~34 clocks
-// against 128 mma.sync of 16).
+// biases start the sums, as products of constant inputs. What bounds it: the chain of
+// four layers (store, products, commit, load: ~700 clocks each), so several blocks share
+// an SM; the products themselves are a sixth of what mma.sync takes (one 128 x 64 x 16
+// product in ~34 clocks against 128 mma.sync of 16).
 #pragma once
 
 #include "mlp.cuh"

@@ -1415,7 +1415,8 @@ __device__ __forceinline__ void step_cell(const StepArgs<Cfg>& A, int x, int y, 
 // A programmatic launch (launch_step) may start while the kernel before it on the
 // stream drains; grid_wait returns when that has finished and its writes are visible to
 // this kernel's ordinary loads (ld_state), and grid_release comes after it.
-// one run: a 2-D grid of blocks over (x, y) and z
+//
+// One run: a 2-D grid of blocks over (x, y) and z.
 template <class Cfg, bool IS3D, int SEED, bool OPEN, int BLOCKS = StepMinBlocks<Cfg, SEED, IS3D>::value>
 __global__ void __launch_bounds__(kStepThreads, BLOCKS)
     step_kernel(const StepArgs<Cfg> A)
